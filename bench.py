@@ -287,7 +287,8 @@ def cpu_oracle_rate(w, seconds: float):
 # Sources of each timed kernel: a recorded DRAM traffic figure stands only
 # while these files are unchanged.
 KERNEL_SOURCES = {
-    "traj_kernel": ("jz_kernels.cu", "jz_traj.cuh", "jz_device.cuh"),
+    "traj_kernel": ("jz_traj2d.cu", "jz_traj3d.cu", "jz_traj_kernel.cuh", "jz_traj.cuh",
+                    "jz_device.cuh"),
     "persistent_kernel": ("jz_batch.cu", "jz_traj.cuh", "jz_device.cuh"),
     "sw_kernel": ("jz_sw.cu", "jz_device.cuh"),
 }

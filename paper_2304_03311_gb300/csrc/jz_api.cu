@@ -171,6 +171,17 @@ void build_tables_into(const jz_params& p, uint32_t tb[4], uint32_t* tcut)
     }
 }
 
+// Whether a switched site's threshold of m > 0 can round up to 2^32 - 1, the
+// value of m <= 0: 2 beta m / den for the smallest m = 1 below 2^-32, doubled
+// for the rounding of the formula.
+int weak_coupling(const jz_params& p)
+{
+    const long long den = p.protocol == 2 && p.d == 3 ? p.n_step / p.L : p.n_step;
+    return 2.0 * p.beta / (double)den < 5e-10;
+}
+
+bool never_flips(const uint32_t tb[4]) { return tb[0] == 0u; }
+
 void build_tables(const jz_params& p, uint32_t tb[4], std::vector<uint32_t>& tcut, size_t off)
 {
     build_tables_into(p, tb, tcut.data() + off);
@@ -260,7 +271,7 @@ jz::LaunchShape shape_for(const jz::Geom& g, int cta_threads)
         const int per_warp = 32 / s.team_threads;
         int warps = (cta_threads > 0 ? cta_threads : 128) / 32;
         if (warps < 1) warps = 1;
-        while (warps > 1 && ((size_t)warps * per_warp * lat > jz::kMaxSmemPerCta ||
+        while (warps > 1 && ((size_t)warps * per_warp * lat + jz::kPairReserve > jz::kMaxSmemPerCta ||
                              warps * per_warp > jz::kMaxTeamsHost))
             --warps;
         s.teams = warps * per_warp;
@@ -540,6 +551,7 @@ int run_group(ising_ctx* ctx, const jz_params* jobs, const std::vector<int>& idx
         J.cta0 = cta;
         if (sw) build_bond_tables(p, J.tb, ctx->h_tcut, off);
         else build_tables(p, J.tb, ctx->h_tcut, off);
+        J.weak = weak_coupling(p);
         J.tcut = d_tcut + off;
         J.w_out = outs_on_device ? (long long*)outs[idx[i]] : (long long*)ctx->work.ptr + traj_off;
         J.spins_out = nullptr;
@@ -626,8 +638,10 @@ int run_group(ising_ctx* ctx, const jz_params* jobs, const std::vector<int>& idx
     } else {
         uint32_t* gS = nullptr;
         if (in_hbm) gS = (uint32_t*)ctx->lattice.ptr;
+        bool never = false;
+        for (int i = 0; i < n_jobs; ++i) never = never || never_flips(ctx->h_jobs[i].tb);
         if ((rc = cuda_err(jz::launch_traj(p0.d, g, K, (const jz::JobDesc*)ctx->jobs.ptr,
-                                           n_jobs, n_cta, sh, st, gS))))
+                                           n_jobs, n_cta, sh, never, st, gS))))
             return rc;
     }
     if ((rc = cuda_err(cudaEventRecord(ctx->ev_k1, st)))) return rc;
@@ -1153,14 +1167,15 @@ extern "C" int ising_bounds_status(unsigned int* sites, unsigned int* index, int
 {
 #ifdef JZ_BOUNDS_CHECK
     if (!sites || !index) return ISING_ERR_ARG;
-    unsigned int a[2], b[2], c[2];
+    unsigned int a[2], b[2], c[2], d[2];
     int rc;
-    if ((rc = cuda_err(jz::bounds_status_traj(a, clear != 0))) ||
+    if ((rc = cuda_err(jz::bounds_status_traj2d(a, clear != 0))) ||
+        (rc = cuda_err(jz::bounds_status_traj3d(d, clear != 0))) ||
         (rc = cuda_err(jz::bounds_status_batch(b, clear != 0))) ||
         (rc = cuda_err(jz::bounds_status_sw(c, clear != 0))))
         return rc;
-    *sites = a[0] | b[0] | c[0];
-    *index = a[0] ? a[1] : b[0] ? b[1] : c[1];
+    *sites = a[0] | b[0] | c[0] | d[0];
+    *index = a[0] ? a[1] : b[0] ? b[1] : c[0] ? c[1] : d[1];
     return ISING_OK;
 #else
     (void)sites;
@@ -1223,6 +1238,7 @@ extern "C" int jarzynski_run_noalloc(const jz_params* p, int64_t* work_int_out, 
     uint32_t* h_tcut = g_noalloc_host + kNoAllocJobBytes / sizeof(uint32_t);
     if (sw) build_bond_tables_into(*p, J.tb, h_tcut);
     else build_tables_into(*p, J.tb, h_tcut);
+    J.weak = weak_coupling(*p);
     J.tcut = d_tcut;
     J.w_out = (long long*)work_int_out;
     J.spins_out = nullptr;
@@ -1241,15 +1257,16 @@ extern "C" int jarzynski_run_noalloc(const jz_params* p, int64_t* work_int_out, 
     if (sw) return cuda_err(jz::launch_sw(p->d, g, K, (const jz::JobDesc*)base, 1, p->n_traj, st));
     const jz::LaunchShape sh = default_shape(p->d, g, p->n_traj);
     return cuda_err(jz::launch_traj(p->d, g, K, (const jz::JobDesc*)base, 1,
-                                    (p->n_traj + sh.teams - 1) / sh.teams, sh, st));
+                                    (p->n_traj + sh.teams - 1) / sh.teams, sh, never_flips(J.tb),
+                                    st));
 }
 
 // --------------------------------------------------- persistent batch plans --
 namespace jz {
-cudaError_t persistent_prepare(size_t smem, int threads, int* blocks_per_sm);
+cudaError_t persistent_prepare(bool pair, size_t smem, int threads, int* blocks_per_sm);
 cudaError_t launch_persistent(const BatchJob* jobs, const int2* items, int n_items,
                               unsigned int* counter, const PhiloxKeys& K, int grid, int threads,
-                              size_t smem, cudaStream_t st);
+                              bool pair, size_t smem, cudaStream_t st);
 cudaError_t launch_estimator_batch(const EstJob* jobs, int n_jobs, double* out, cudaStream_t st);
 }  // namespace jz
 
@@ -1285,6 +1302,7 @@ struct jz_plan {
     ising_ctx* ctx = nullptr;
     int n_jobs = 0, n_items = 0, threads = 0, grid = 0;
     size_t smem = 0;
+    bool pair = true;   // the acceptance table fits and serves every job
     jz::PhiloxKeys K{};
     DevBuf jobs, items, tcut, counter, est_jobs;
     double* est_out = nullptr;
@@ -1438,6 +1456,8 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
         J.traj0 = p.traj0;
         J.cta0 = 0;
         build_tables(p, J.tb, tcut, toff[j]);
+        J.weak = weak_coupling(p);
+        pl->pair = pl->pair && !never_flips(J.tb) && jz::traj_pairs(B.g, B.sh.teams, false);
         J.w_out = (long long*)work_outs[j];
         J.spins_out = nullptr;
         if (sw_therm(p)) {
@@ -1492,7 +1512,7 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
                          return a.first > b.first;
                      });
     pl->n_items = (int)items.size();
-    pl->smem = smem;
+    pl->smem = smem + (pl->pair ? jz::kPairTable * sizeof(uint2) : 0);
     int rc;
     if ((rc = ensure(ctx, pl->tcut, tcut.size() * sizeof(uint32_t))) ||
         (rc = ensure(ctx, pl->jobs, bj.size() * sizeof(jz::BatchJob))) ||
@@ -1579,7 +1599,7 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
     }
     int per_sm = 0;
     cudaDeviceProp prop;
-    if ((rc = cuda_err(jz::persistent_prepare(smem, cta, &per_sm))) ||
+    if ((rc = cuda_err(jz::persistent_prepare(pl->pair, pl->smem, cta, &per_sm))) ||
         (rc = cuda_err(cudaGetDeviceProperties(&prop, ctx->device)))) {
         plan_release(pl);
         return rc;
@@ -1617,7 +1637,7 @@ int plan_enqueue(jz_plan* pl)
         if ((rc = cuda_err(jz::launch_persistent((const jz::BatchJob*)pl->jobs.ptr,
                                                  (const int2*)pl->items.ptr, pl->n_items,
                                                  (unsigned int*)pl->counter.ptr, pl->K, pl->grid,
-                                                 pl->threads, pl->smem, st))))
+                                                 pl->threads, pl->pair, pl->smem, st))))
             return rc;
     }
     for (const auto& G : pl->sw)

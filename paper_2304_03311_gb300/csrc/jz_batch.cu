@@ -17,9 +17,9 @@ namespace jz {
 
 constexpr int kMaxTeams = 64;
 
-template <int D, bool FAST, class Bar>
+template <int D, bool FAST, bool PAIR, class Bar>
 __device__ __forceinline__ void run_item(const BatchJob& B, const PhiloxKeys& K, int traj_lo,
-                                         uint32_t* S, const uint32_t* tab, int* s_work, Bar bar)
+                                         uint32_t* S, const uint2* tab, int* s_work, Bar bar)
 {
     const TeamJob tj = team_job(B.J, B.g.Ly);
     int team, tid;
@@ -34,7 +34,7 @@ __device__ __forceinline__ void run_item(const BatchJob& B, const PhiloxKeys& K,
     const long long V = (long long)B.g.nrep * B.g.Lt * B.g.Ly * B.g.L;
     // therm_update = 1: the job starts from its thermalised spins
     const int8_t* sin = (has && tj.start_in) ? B.J.spins_in + local * V : nullptr;
-    const int dE = run_trajectory<D, FAST, 0, 0>(B.g, K, tj, B.J.traj0 + local, St, tab, tid,
+    const int dE = run_trajectory<D, FAST, PAIR, false, 0, 0>(B.g, K, tj, B.J.traj0 + local, St, tab, tid,
                                                  B.sh.team_threads, bar, sin);
     if (has && dE != 0) atomicAdd(&s_work[tm], dE);
     __syncthreads();
@@ -47,22 +47,24 @@ __device__ __forceinline__ void run_item(const BatchJob& B, const PhiloxKeys& K,
                         tid, B.sh.team_threads);
 }
 
-template <int D, bool FAST>
+template <int D, bool FAST, bool PAIR>
 __device__ __forceinline__ void run_item_any(const BatchJob& B, const PhiloxKeys& K, int traj_lo,
-                                             uint32_t* S, const uint32_t* tab, int* s_work)
+                                             uint32_t* S, const uint2* tab, int* s_work)
 {
-    if (B.sh.warp) run_item<D, FAST>(B, K, traj_lo, S, tab, s_work, WarpBarrier{});
-    else run_item<D, FAST>(B, K, traj_lo, S, tab, s_work, CtaBarrier{});
+    if (B.sh.warp) run_item<D, FAST, PAIR>(B, K, traj_lo, S, tab, s_work, WarpBarrier{});
+    else run_item<D, FAST, PAIR>(B, K, traj_lo, S, tab, s_work, CtaBarrier{});
 }
 
+template <bool PAIR>
 __global__ void __launch_bounds__(512)
 persistent_kernel(const BatchJob* __restrict__ jobs, const int2* __restrict__ items, int n_items,
                   unsigned int* __restrict__ counter, const PhiloxKeys K)
 {
-    extern __shared__ uint32_t S[];
+    extern __shared__ uint2 s_dyn[];
+    uint2* s_tab = s_dyn;
+    uint32_t* S = (uint32_t*)(s_dyn + (PAIR ? kPairTable : 0));
     __shared__ int s_item;
     __shared__ int s_work[kMaxTeams];
-    __shared__ uint32_t s_tab[8];
     for (;;) {
         if (threadIdx.x == 0) s_item = (int)atomicAdd(counter, 1u);
         __syncthreads();
@@ -70,16 +72,18 @@ persistent_kernel(const BatchJob* __restrict__ jobs, const int2* __restrict__ it
         if (it >= n_items) break;
         const int2 item = items[it];
         const BatchJob& B = jobs[item.x];
-        if (threadIdx.x < 8)
-            s_tab[threadIdx.x] = threadIdx.x < (unsigned)B.D ? B.J.tb[threadIdx.x] : 0u;
-        if (threadIdx.x < kMaxTeams) s_work[threadIdx.x] = 0;
+        if (PAIR) {
+            if (B.D == 2) fill_pairs<2>(s_tab, B.J.tb);
+            else fill_pairs<3>(s_tab, B.J.tb);
+        }
+        for (int i = threadIdx.x; i < kMaxTeams; i += blockDim.x) s_work[i] = 0;
         __syncthreads();
         if (B.D == 2) {
-            if (B.fast) run_item_any<2, true>(B, K, item.y, S, s_tab, s_work);
-            else run_item_any<2, false>(B, K, item.y, S, s_tab, s_work);
+            if (B.fast) run_item_any<2, true, PAIR>(B, K, item.y, S, s_tab, s_work);
+            else run_item_any<2, false, PAIR>(B, K, item.y, S, s_tab, s_work);
         } else {
-            if (B.fast) run_item_any<3, true>(B, K, item.y, S, s_tab, s_work);
-            else run_item_any<3, false>(B, K, item.y, S, s_tab, s_work);
+            if (B.fast) run_item_any<3, true, PAIR>(B, K, item.y, S, s_tab, s_work);
+            else run_item_any<3, false, PAIR>(B, K, item.y, S, s_tab, s_work);
         }
         __syncthreads();   // shared memory and s_item are reused by the next item
     }
@@ -125,29 +129,29 @@ estimator_batch_kernel(const EstJob* __restrict__ jobs, double* __restrict__ out
 // The attribute is set to the per-CTA maximum (not this plan's size) so that
 // graphs captured for larger plans stay launchable after smaller ones; the
 // kernel's static shared memory comes out of the same opt-in limit.
-cudaError_t persistent_prepare(size_t smem, int threads, int* blocks_per_sm)
+cudaError_t persistent_prepare(bool pair, size_t smem, int threads, int* blocks_per_sm)
 {
+    const auto kern = pair ? persistent_kernel<true> : persistent_kernel<false>;
     int dev = 0, optin = 0;
     cudaFuncAttributes fa;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, persistent_kernel);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
     if (e != cudaSuccess) return e;
     const int max_dyn = optin - (int)fa.sharedSizeBytes;
     if ((long long)smem > max_dyn) return cudaErrorInvalidValue;
-    e = cudaFuncSetAttribute(persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             max_dyn);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, max_dyn);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, persistent_kernel,
-                                                          threads, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, threads, smem);
 }
 
 cudaError_t launch_persistent(const BatchJob* jobs, const int2* items, int n_items,
                               unsigned int* counter, const PhiloxKeys& K, int grid, int threads,
-                              size_t smem, cudaStream_t st)
+                              bool pair, size_t smem, cudaStream_t st)
 {
-    persistent_kernel<<<grid, threads, smem, st>>>(jobs, items, n_items, counter, K);
+    const auto kern = pair ? persistent_kernel<true> : persistent_kernel<false>;
+    kern<<<grid, threads, smem, st>>>(jobs, items, n_items, counter, K);
     return cudaGetLastError();
 }
 

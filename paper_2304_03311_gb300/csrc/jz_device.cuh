@@ -11,11 +11,16 @@
 // shifted by one nibble (the other x neighbour).  Two Philox4x32-10 blocks
 // give the eight acceptance words of one spin word.
 #pragma once
+#include <cstddef>
 #include <cstdint>
 
 namespace jz {
 
 constexpr int kMaxJobsPerLaunch = 4096;
+constexpr int kPairTable = 256;   // entries of the acceptance table of site pairs
+constexpr size_t kMaxDynSmem = 227 * 1024;   // shared memory of one CTA
+// Kept free beside the lattices for that table and the kernels' static arrays.
+constexpr size_t kPairReserve = kPairTable * 8 + 512;
 
 // Bounds-checked builds (compiled with -DJZ_BOUNDS_CHECK: the debug library).
 // Every lattice access of the trajectory kernels and every label / spin-bit
@@ -87,6 +92,7 @@ struct JobDesc {
     long long cta0;     // first CTA of the job in the launch grid
     uint32_t tb[4];     // bulk thresholds by anti-aligned neighbour count a:
                         // tb[a] = T(m = 2D - 2a), a < D
+    int weak;           // 1: a threshold of tcut with m > 0 may round up to 2^32 - 1
     const uint32_t* tcut;   // [n_step][8D] switched-site thresholds
     long long* w_out;       // [n_traj] W_int
     int8_t* spins_out;      // [n_traj][V] final spins (+-1) or nullptr
@@ -128,19 +134,13 @@ __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, u
     return make_uint4(c0, c1, c2, c3);
 }
 
-// One block with round 0's two products supplied: p0 = M0 * c0 and
-// (hi1, lo1) = M1 * c2.  Counter word 2 is the trajectory index, fixed for a
-// whole trajectory, and successive blocks of a thread step c0 by a constant,
-// so callers form p0 by 64-bit additions instead of a wide multiply.
-__device__ __forceinline__ uint4 philox_p0(uint64_t p0, uint32_t c1, uint32_t hi1, uint32_t lo1,
-                                           uint32_t c3, const PhiloxKeys& K)
+// The block whose counter entering round R is (c0, c1, c2, c3).
+template <int R>
+__device__ __forceinline__ uint4 philox_from(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                             const PhiloxKeys& K)
 {
-    uint32_t c0 = hi1 ^ c1 ^ K.k0[0];
-    uint32_t c2 = (uint32_t)(p0 >> 32) ^ c3 ^ K.k1[0];
-    c1 = lo1;
-    c3 = (uint32_t)p0;
 #pragma unroll
-    for (int i = 1; i < 10; ++i) {
+    for (int i = R; i < 10; ++i) {
         const uint64_t q0 = (uint64_t)kPhiloxM0 * c0;
         const uint64_t q1 = (uint64_t)kPhiloxM1 * c2;
         const uint32_t n0 = (uint32_t)(q1 >> 32) ^ c1 ^ K.k0[i];
@@ -153,11 +153,14 @@ __device__ __forceinline__ uint4 philox_p0(uint64_t p0, uint32_t c1, uint32_t hi
     return make_uint4(c0, c1, c2, c3);
 }
 
-// The same block with only round 0's product M1 * c2 supplied (hi1, lo1).
+// One block with round 0's product (hi1, lo1) = M1 * c2 supplied: counter word
+// 2 is the trajectory index, fixed for a whole trajectory.
 __device__ __forceinline__ uint4 philox_r0(uint32_t c0, uint32_t c1, uint32_t hi1, uint32_t lo1,
                                            uint32_t c3, const PhiloxKeys& K)
 {
-    return philox_p0((uint64_t)kPhiloxM0 * c0, c1, hi1, lo1, c3, K);
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * c0;
+    return philox_from<1>(hi1 ^ c1 ^ K.k0[0], lo1, (uint32_t)(p0 >> 32) ^ c3 ^ K.k1[0],
+                          (uint32_t)p0, K);
 }
 
 // The last stage of the FP64 estimator of one job (Appendix A, eq.

@@ -21,10 +21,14 @@
 namespace jz {
 size_t traj_smem_bytes(const Geom& g);
 // gS: nullptr to keep the lattices in shared memory, else an HBM buffer of
-// n_cta * sh.teams * 2 * NR * GW words, one slice per CTA.
+// n_cta * sh.teams * 2 * NR * GW words, one slice per CTA.  never: a job has a
+// bulk threshold of 0 (jzh::never_flips), which the acceptance table cannot hold.
 cudaError_t launch_traj(int D, const Geom& g, const PhiloxKeys& K, const JobDesc* jobs,
-                        int n_jobs, long long n_cta, const LaunchShape& sh, cudaStream_t st,
-                        uint32_t* gS = nullptr);
+                        int n_jobs, long long n_cta, const LaunchShape& sh, bool never,
+                        cudaStream_t st, uint32_t* gS = nullptr);
+// Whether the acceptance table fits beside `teams` lattices g in shared memory
+// (hbm: beside none); without it the kernel counts thresholds (jz_traj.cuh).
+bool traj_pairs(const Geom& g, int teams, bool hbm);
 // CTAs of shape sh resident per SM for the trajectory kernel launch_traj
 // runs on g with its lattices in shared memory.
 cudaError_t traj_occupancy(int D, const Geom& g, const LaunchShape& sh, int* ctas_per_sm);
@@ -45,7 +49,8 @@ double run_probe(int kind, int device);
 // Status words of the bounds-checked build, one per translation unit with
 // kernels (zeros in release builds): [0] = check sites that saw an index
 // outside their array, [1] = one such index; clear resets them.
-cudaError_t bounds_status_traj(unsigned int out[2], bool clear);
+cudaError_t bounds_status_traj2d(unsigned int out[2], bool clear);
+cudaError_t bounds_status_traj3d(unsigned int out[2], bool clear);
 cudaError_t bounds_status_batch(unsigned int out[2], bool clear);
 cudaError_t bounds_status_sw(unsigned int out[2], bool clear);
 cudaError_t plain_trajectory(int D, const Geom& g, const PhiloxKeys& K, int l, int dir,
@@ -53,7 +58,7 @@ cudaError_t plain_trajectory(int D, const Geom& g, const PhiloxKeys& K, int l, i
                              const uint32_t tb[4], const uint32_t* tcut, int8_t* s,
                              long long* w, cudaStream_t st);
 constexpr int kMaxJackBlocksHost = 64;
-constexpr size_t kMaxSmemPerCta = 227 * 1024;
+constexpr size_t kMaxSmemPerCta = kMaxDynSmem;
 constexpr int kMaxTeamsHost = 64;   // teams per CTA
 }  // namespace jz
 
@@ -110,6 +115,9 @@ void build_tables(const jz_params& p, uint32_t tb[4], std::vector<uint32_t>& tcu
 // The same tables written to tcut[0 .. n_step * 8d) (bond tables: n_step * 2).
 void build_tables_into(const jz_params& p, uint32_t tb[4], uint32_t* tcut);
 void build_bond_tables_into(const jz_params& p, uint32_t tb[4], uint32_t* tcut);
+int weak_coupling(const jz_params& p);
+// Whether a site may never flip: a bulk threshold of 0 (strong couplings).
+bool never_flips(const uint32_t tb[4]);
 uint32_t bond_threshold(double x);
 void step_weights(const jz_params& p, long long k, long long* den, long long* w_self,
                   long long* w_glue);

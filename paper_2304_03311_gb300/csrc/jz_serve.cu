@@ -186,6 +186,7 @@ int jz_server::launch(Slot& s, Job& j)
     std::memset(&J, 0, sizeof J);
     if (p.update == 1) build_bond_tables(p, J.tb, s.tcut, 0);
     else build_tables(p, J.tb, s.tcut, 0);
+    J.weak = weak_coupling(p);
     std::memcpy(s.h_tcut, s.tcut.data(), n_tcut * sizeof(uint32_t));
     char* d = nullptr;
     if ((rc = cuda_err(cudaMallocAsync((void**)&d, j.need, s.stream)))) return rc;
@@ -244,7 +245,7 @@ int jz_server::launch(Slot& s, Job& j)
                            ? jz::launch_sw(p.d, g, K, d_desc, 1, p.n_traj, s.stream)
                            : jz::launch_traj(p.d, g, K, d_desc, 1,
                                              (p.n_traj + sh.teams - 1) / sh.teams, sh,
-                                             s.stream))) ||
+                                             never_flips(J.tb), s.stream))) ||
         (rc = cuda_err(jz::launch_estimator(d_work, p.n_traj, p.beta / (double)p.n_step,
                                             p.direction, B, d_est, s.stream))) ||
         (rc = cuda_err(cudaMemcpyAsync(s.h_est, d_est, 3 * sizeof(double),

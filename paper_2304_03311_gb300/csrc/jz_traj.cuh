@@ -11,17 +11,32 @@
 // nibble j (bits 4j..4j+3) of word q is the colour-c site h = 8q + j of the
 // row, x = 2h + p, p = (c + t + y) mod 2, value 0 for spin +1 and 1 for -1.
 // A word's eight sites draw from Philox blocks 2q and 2q+1 of their row.
-// Nibble-wise sums of XORs give the anti-aligned neighbour count of all eight
-// sites at once (at most 6 < 16, so no carries cross nibbles).
+// Nibble-wise sums of the neighbours' words give the number of neighbours of
+// spin -1 of all eight sites at once (at most 6, so no carries cross nibbles).
 //
 // Team mapping: a team of GW * L_y * TS * RS threads; thread (r0, t0, y, q)
-// owns word q of row y of the time slices t0, t0 + TS, ... in the replicas
-// r0, r0 + RS, ... and both colours, so all its index and wrap arithmetic is
-// fixed.  RS > 1 only when TS = L_t (a whole time column per thread slot):
-// lattices so small that one replica's words leave most of a warp idle.  Rows t >= 2 take the bulk
-// path; the rows t = 0, 1 next to the cut blend in the glued replica and
-// handle the switched column x = l.  CW, CLY > 0 fix GW and L_y at compile
-// time (neighbour loads then use immediate offsets); 0 reads them from Geom.
+// owns word q of row y of every TS-th time slice in the replicas r0, r0 + RS,
+// ... and both colours, so all its index and wrap arithmetic is fixed.  RS > 1
+// only when TS = L_t (a whole time column per thread slot): lattices so small
+// that one replica's words leave most of a warp idle.  A replica's rows are one
+// or two edge rows, which blend in the glued replica and handle the switched
+// columns (half_sweep says which rows), and bulk rows.  CW, CLY > 0 fix GW and
+// L_y at compile time (neighbour loads then use immediate offsets); 0 reads
+// them from Geom.
+//
+// What bounds it (ncu and instruction-mix probes on GB300, cycles per SM
+// sub-partition and spin word of 32 lanes): the pipes that issue the two
+// Philox blocks of a word and its update.  A 32 x 32 -> 64-bit multiply holds
+// the FMA pipe for 4 cycles and a result port that it shares with the 2-cycle
+// logic and add instructions for 2; the bare Philox of a word (34 multiplies, 38
+// three-input XORs) takes 143 cycles, every further ALU instruction adds about
+// 1.8, every multiply-add 1.4, every shared load about 1.  So the update is
+// written for few instructions of any kind: thresholds looked up for two sites
+// at once, sums instead of XORs, one funnel shift per word, wrap-free bulk rows.
+// 2D L = 64: 134 instructions and 230 cycles per word (158 and 311 with one
+// lookup per site, four copies of the half-sweep whose code overflowed the
+// instruction cache, and a cut pass that recomputed its geometry):
+// 1.07e12 -> 1.53e12 spin updates/s on a scan of 31 x 1024 trajectories.
 //
 // The work increment is gathered inside the first colour-0 half-sweep of each
 // step: for every (r, y) exactly one of the switched sites (l, y, 0)^r and
@@ -37,28 +52,101 @@
 
 namespace jz {
 
-// Flip bits (bit 4j) of the eight sites of a word.  dsum nibble j = a_j, the
-// number of anti-aligned neighbours of site j (energy cost m = 2D - 2 a_j);
-// tab[a] = T(m) for a < D.  Sites with a_j >= D (m <= 0) always flip.  Sites
-// 0..3 use the words of block ua, sites 4..7 those of block ub.
-template <int D>
-__device__ __forceinline__ uint32_t accept8(uint32_t dsum, const uint4& ua, const uint4& ub,
-                                            const uint32_t* tab)
+
+// ------------------------------------------------------------- acceptance --
+// A site with a anti-aligned neighbours (energy cost m = 2D - 2a) flips when
+// a >= D, else iff its draw is below tb[a] = T(m).
+
+// f += 2^SH if u <= t: one compare and one predicated add.
+template <int SH>
+__device__ __forceinline__ void add_if_le(uint32_t& f, uint32_t u, uint32_t t)
 {
-    uint32_t f = ((dsum + (uint32_t)(8 - D) * 0x11111111u) >> 3) & 0x11111111u;
-    const uint32_t ev = (dsum & 0x0F0F0F0Fu) << 2;   // sites 0,2,4,6: byte offsets into tab
-    const uint32_t od = (dsum >> 2) & 0x3C3C3C3Cu;   // sites 1,3,5,7
-    const unsigned char* tb = reinterpret_cast<const unsigned char*>(tab);
-    auto T = [&](uint32_t off) { return *reinterpret_cast<const uint32_t*>(tb + off); };
-    if (ua.x < T(ev & 0xFFu)) f |= 1u;
-    if (ua.y < T(od & 0xFFu)) f |= 1u << 4;
-    if (ua.z < T(__byte_perm(ev, 0, 0x4441))) f |= 1u << 8;
-    if (ua.w < T(__byte_perm(od, 0, 0x4441))) f |= 1u << 12;
-    if (ub.x < T(__byte_perm(ev, 0, 0x4442))) f |= 1u << 16;
-    if (ub.y < T(__byte_perm(od, 0, 0x4442))) f |= 1u << 20;
-    if (ub.z < T(__byte_perm(ev, 0, 0x4443))) f |= 1u << 24;
-    if (ub.w < T(__byte_perm(od, 0, 0x4443))) f |= 1u << 28;
+    asm("{.reg .pred q; setp.le.u32 q, %1, %2; @q add.u32 %0, %0, %3;}"
+        : "+r"(f)
+        : "r"(u), "r"(t), "n"((int)(1u << SH)));
+}
+// f += 2^SH if u < t.
+template <int SH>
+__device__ __forceinline__ void add_if_lt(uint32_t& f, uint32_t u, uint32_t t)
+{
+    asm("{.reg .pred q; setp.lt.u32 q, %1, %2; @q add.u32 %0, %0, %3;}"
+        : "+r"(f)
+        : "r"(u), "r"(t), "n"((int)(1u << SH)));
+}
+
+// PAIR acceptance, the form of every job that allows it: a 256-entry table of threshold pairs in shared memory,
+// indexed by one byte of v, i.e. by two sites at once.  Nibble j of v is site
+// j's state: its neighbours of spin -1 counted (at most 2D < 8), its own spin in
+// bit 3.  A site flips iff its draw is at most its threshold.  Returns the flip
+// bits (bit 4j); sites 0..3 use the words of block ua, sites 4..7 those of ub.
+__device__ __forceinline__ uint32_t accept_pairs(uint32_t v, const uint4& ua, const uint4& ub,
+                                                 const uint2* tab)
+{
+    const uint2 t01 = tab[v & 0xFFu];
+    const uint2 t23 = tab[__byte_perm(v, 0, 0x4441)];
+    const uint2 t45 = tab[__byte_perm(v, 0, 0x4442)];
+    const uint2 t67 = tab[v >> 24];
+    uint32_t f = 0;
+    add_if_le<0>(f, ua.x, t01.x);
+    add_if_le<4>(f, ua.y, t01.y);
+    add_if_le<8>(f, ua.z, t23.x);
+    add_if_le<12>(f, ua.w, t23.y);
+    add_if_le<16>(f, ub.x, t45.x);
+    add_if_le<20>(f, ub.y, t45.y);
+    add_if_le<24>(f, ub.z, t67.x);
+    add_if_le<28>(f, ub.w, t67.y);
     return f;
+}
+
+// The table of one job, filled by the CTA's threads: "at most tb[a] - 1", or
+// "always" (a >= D).  It cannot say "never" (tb[a] = 0, strong couplings): such
+// jobs take the counts below.
+template <int D>
+__device__ __forceinline__ void fill_pairs(uint2* tab, const uint32_t* __restrict__ tb)
+{
+    auto at = [&](int v) {
+        const int s = v & 7;
+        const int a = (v & 8) ? 2 * D - s : s;
+        if (a < 0 || a >= D) return 0xFFFFFFFFu;
+        return __ldg(tb + a) - 1u;
+    };
+    for (int i = threadIdx.x; i < kPairTable; i += blockDim.x)
+        tab[i] = make_uint2(at(i & 15), at(i >> 4));
+}
+
+// COUNT acceptance, for jobs without a table (a threshold of zero, or no shared
+// memory left beside the lattice) and for run_rows, where the counts are off the
+// path from one half-sweep to the next: 2D, 4 instructions per site against the
+// table's 3.5 (3D: 6).  Nibble j of the result is the number of thresholds T[i],
+// i < D, above site j's draw.  tb grows with a, so the site flips iff
+// a + count >= D.  It depends on the draws alone.
+template <int D>
+__device__ __forceinline__ uint32_t count8(const uint4& ua, const uint4& ub, const uint32_t* T)
+{
+    uint32_t n = 0;
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+        add_if_lt<0>(n, ua.x, T[i]);
+        add_if_lt<4>(n, ua.y, T[i]);
+        add_if_lt<8>(n, ua.z, T[i]);
+        add_if_lt<12>(n, ua.w, T[i]);
+        add_if_lt<16>(n, ub.x, T[i]);
+        add_if_lt<20>(n, ub.y, T[i]);
+        add_if_lt<24>(n, ub.z, T[i]);
+        add_if_lt<28>(n, ub.w, T[i]);
+    }
+    return n;
+}
+
+// The flip bits from the counts n, the nibble-wise sums s of the neighbours of
+// spin -1 and the own spins: with a = s (own 0) or 2D - s (own 1), the new
+// spin is [s + n >= D] or [s - n >= D + 1], and 3 - n = n ^ 3, so both are
+// bit 3 of one nibble-wise sum (between 1 and 14: no carries).
+template <int D>
+__device__ __forceinline__ uint32_t flips_of_counts(uint32_t s, uint32_t own, uint32_t n)
+{
+    const uint32_t x = s + (n ^ (own * 3u)) - own * 4u + (uint32_t)(8 - D) * 0x11111111u;
+    return ((x >> 3) & 0x11111111u) ^ own;
 }
 
 __device__ __forceinline__ uint32_t word8(const uint4& ua, const uint4& ub, int j)
@@ -75,47 +163,109 @@ struct TeamJob {
     int prot;     // 1: every switched column together; 2: one column y at a time
     int den;      // steps of one column's run: N (protocol 1), N / L_y (protocol 2)
     const uint32_t* tcut;
+    uint32_t tb[3];       // bulk thresholds, a < D
+    bool weak;            // a switched threshold of m > 0 may round up to 2^32 - 1
+};
+
+// What a row's update needs beside its words: the protocol step (k < 0: none)
+// and its weights.
+struct StepState {
+    int k, lg, w_self, w_glue;
+    const uint32_t* tk;   // step k's switched-site thresholds
+    bool record;
+};
+
+// Where a team's lattice lies: byte addresses of its words, 32-bit ones in
+// shared memory (one add per address, immediate offsets folded into the
+// access) or pointers into an HBM slice.
+template <bool HBM>
+struct Mem;
+template <>
+struct Mem<false> {
+    using A = uint32_t;
+    static __device__ __forceinline__ A at(uint32_t* p)
+    {
+        return (uint32_t)__cvta_generic_to_shared(p);
+    }
+    static __device__ __forceinline__ uint32_t ld(A a)
+    {
+        uint32_t v;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+        return v;
+    }
+    static __device__ __forceinline__ void st(A a, uint32_t v)
+    {
+        asm volatile("st.shared.u32 [%0], %1;" : : "r"(a), "r"(v) : "memory");
+    }
+};
+template <>
+struct Mem<true> {
+    using A = char*;
+    static __device__ __forceinline__ A at(uint32_t* p) { return (char*)p; }
+    static __device__ __forceinline__ uint32_t ld(A a) { return *(const uint32_t*)a; }
+    static __device__ __forceinline__ void st(A a, uint32_t v) { *(uint32_t*)a = v; }
 };
 
 // CLT, CTS > 0: L_t and the slice step TS fixed at compile time (the 2D L = 64,
 // L_t = 64 warp teams); 0 reads them from Geom and the team size.
-template <int D, bool FAST, int CW = 0, int CLY = 0, int CLT = 0, int CTS = 0>
+template <int D, bool FAST, bool PAIR, bool HBM, int CW = 0, int CLY = 0, int CLT = 0, int CTS = 0>
 struct Traj {
+    using M = Mem<HBM>;
+    using A = typename M::A;
+    // A thread's edge row (t = 0, 1 next to the cut, or any other, whose
+    // neighbour "across" is its t + 1 row): byte offsets that hold for a whole
+    // trajectory.
+    struct Edge {
+        int t;            // the row
+        int n, x;         // the ordinary time neighbour; the row across
+        int g, gw, rw;    // the glued partner across: + g, in replica rw + gw
+    };
+
     const Geom& g;
     uint32_t* S;              // this team's spin words [2][NR * GW]
-    const uint32_t* tab;      // shared bulk thresholds
+    A S0;                     // their address
+    const uint2* tab;         // PAIR: the job's threshold pairs
+    const TeamJob& J;
     const PhiloxKeys& K;
     uint32_t hi1, lo1;        // M1 * traj: round 0 of Philox for counter word 2
     uint32_t c3base;          // dir bit << 1 | l << 2
     int q, y, t0, TS;         // this thread's word, row y, first slice and slice step
     int r0, RS;               // first replica and replica step
-    int d_qm, d_qp;           // word offset of the x-shift neighbour word (p = 0 / 1)
-    int d_ym, d_yp;           // word offsets of the rows y-1 / y+1 (3D)
+    int d_qm, d_qp;           // byte offset of the x-shift neighbour word (p = 0 / 1)
+    int d_ym, d_yp;           // byte offsets of the rows y-1 / y+1 (3D)
+    Edge edge;                // TS >= 3: the first row of each replica
+    int tb, n_bulk, up_last;  // first bulk row, their number, the last one's t + 1 row
     uint32_t vmask;           // nibbles of word q that hold sites (ragged rows)
     int sh_next, sh_prev;     // ragged rows: nibble position of the wrapped x neighbour
-    uint32_t m_next;
 
     __device__ __forceinline__ int W() const { return CW > 0 ? CW : g.GW; }
-
-    // Word i of one colour's NR * GW lattice words (checked in bounds-checked
-    // builds: an index outside the colour is recorded and the access skipped).
-    __device__ __forceinline__ uint32_t ld(const uint32_t* colour, int i, int site) const
-    {
-        return in_bounds(i, (long long)g.NR * g.GW, site) ? colour[i] : 0u;
-    }
-    __device__ __forceinline__ void st(uint32_t* colour, int i, uint32_t v, int site) const
-    {
-        if (in_bounds(i, (long long)g.NR * g.GW, site)) colour[i] = v;
-    }
     __device__ __forceinline__ int Ly() const { return D == 2 ? 1 : (CLY > 0 ? CLY : g.Ly); }
     __device__ __forceinline__ int rowW() const { return Ly() * W(); }
+    __device__ __forceinline__ int Lt() const { return CLT > 0 ? CLT : g.Lt; }
+    // Philox blocks per row: full words have two each
+    __device__ __forceinline__ int G() const { return CW > 0 && FAST ? 2 * CW : g.G; }
+    __device__ __forceinline__ int step() const { return CTS > 0 ? CTS : TS; }
+
+    // The word at address a, of the colour starting at base (checked in
+    // bounds-checked builds: a word outside the colour is recorded and the
+    // access skipped).
+    __device__ __forceinline__ uint32_t ld(A base, A a, int site) const
+    {
+        return in_bounds((long long)(a - base) >> 2, (long long)g.NR * g.GW, site) ? M::ld(a) : 0u;
+    }
+    __device__ __forceinline__ void st(A base, A a, uint32_t v, int site) const
+    {
+        if (in_bounds((long long)(a - base) >> 2, (long long)g.NR * g.GW, site)) M::st(a, v);
+    }
+    __device__ __forceinline__ A colour(int c) const { return S0 + c * (g.nrep * Lt() * rowW() * 4); }
 
     // tid < 0: a thread with no sites (it still takes part in the barriers).
-    __device__ __forceinline__ Traj(const Geom& g_, uint32_t* S_, const uint32_t* tab_,
-                                    const PhiloxKeys& K_, uint32_t traj, uint32_t c3base_,
+    __device__ __forceinline__ Traj(const Geom& g_, uint32_t* S_, const uint2* tab_,
+                                    const TeamJob& J_, const PhiloxKeys& K_, uint32_t traj,
                                     int tid, int nthr)
-        : g(g_), S(S_), tab(tab_), K(K_), c3base(c3base_)
+        : g(g_), S(S_), S0(M::at(S_)), tab(tab_), J(J_), K(K_)
     {
+        c3base = ((uint32_t)(J.dir < 0) << 1) | ((uint32_t)J.l << 2);
         const uint64_t p1 = (uint64_t)kPhiloxM1 * traj;
         hi1 = (uint32_t)(p1 >> 32);
         lo1 = (uint32_t)p1;
@@ -133,16 +283,33 @@ struct Traj {
             t0 = (tid / col) % TS;
             r0 = (tid / col) / TS;
         }
-        d_qm = (q == 0 ? W() - 1 : q - 1) - q;
-        d_qp = (q == W() - 1 ? 0 : q + 1) - q;
-        d_ym = ((y == 0 ? Ly() - 1 : y - 1) - y) * W();
-        d_yp = ((y == Ly() - 1 ? 0 : y + 1) - y) * W();
+        d_qm = 4 * ((q == 0 ? W() - 1 : q - 1) - q);
+        d_qp = 4 * ((q == W() - 1 ? 0 : q + 1) - q);
+        d_ym = 4 * ((y == 0 ? Ly() - 1 : y - 1) - y) * W();
+        d_yp = 4 * ((y == Ly() - 1 ? 0 : y + 1) - y) * W();
         const int nv = g.Lh - 8 * q;                       // sites in this word
         const int nv_last = g.Lh - 8 * (W() - 1);          // sites in the row's last word
         vmask = nv >= 8 ? 0xFFFFFFFFu : ((1u << (4 * nv)) - 1u);
         sh_next = 4 * ((nv >= 8 ? 8 : nv) - 1);
-        m_next = (1u << sh_next) - 1u;
         sh_prev = q == 0 ? 4 * (nv_last - 1) : 28;
+        const bool rot = step() >= 3;
+        edge = edge_of(!rot ? t0 : t0 == 0 ? Lt() - 1 : t0 - 1);
+        tb = rot ? t0 - 1 + step() : (step() == 1 ? 2 : t0 + 2);
+        const int end = rot ? Lt() - 1 : Lt();
+        n_bulk = tb < end ? (end - tb - 1) / step() + 1 : 0;
+        up_last = 4 * rowW() *
+                  (!rot && tb + (n_bulk - 1) * step() == Lt() - 1 ? -(Lt() - 1) : 1);
+    }
+
+    // Flip bits of a word: s = nibble-wise sums of the neighbours of spin -1.
+    __device__ __forceinline__ uint32_t flips(uint32_t s, uint32_t own, const uint4& ua,
+                                              const uint4& ub) const
+    {
+        if constexpr (PAIR) {
+            return accept_pairs(s + own * 8u, ua, ub, tab);
+        } else {
+            return flips_of_counts<D>(s, own, count8<D>(ua, ub, J.tb));
+        }
     }
 
     // Glue mask: nibbles of word q (row parity p) whose site has x < lg.
@@ -153,225 +320,240 @@ struct Traj {
         return nj == 8 ? 0xFFFFFFFFu : ((1u << (4 * nj)) - 1u);
     }
 
-    // The x neighbour not at the same h: h-1 for p = 0, h+1 for p = 1.  Word w
-    // of the other colour oth is word q of the row; the row's other words are
-    // w + d_qm / w + d_qp.
-    __device__ __forceinline__ uint32_t xshift(const uint32_t* oth, int w, int p,
-                                               uint32_t nx0) const
+    // The x neighbour not at the same h -- h - 1 for p = 0, h + 1 for p = 1 -- of
+    // a word's eight sites, out of two words of the other colour's row: lo (at
+    // offset a) shifted down by s, joined by hi (at offset b) above it.
+    struct XShift {
+        int a, b;
+        uint32_t s, m;   // FAST: a funnel shift by s; ragged: (lo >> s) + hi m
+    };
+    __device__ __forceinline__ XShift xshift(int p) const
     {
-        const uint32_t nb = ld(oth, w + (p ? d_qp : d_qm), 6);
-        if (FAST) return p ? __funnelshift_r(nx0, nb, 4) : __funnelshift_l(nb, nx0, 4);
-        // ragged rows: the row's last word holds fewer than eight sites
-        return p ? (((nx0 >> 4) & m_next) | ((nb & 0xFu) << sh_next))
-                 : ((nx0 << 4) | ((nb >> sh_prev) & 0xFu));
+        XShift x;
+        x.a = p ? 0 : d_qm;
+        x.b = p ? d_qp : 0;
+        if (FAST) {
+            x.s = p ? 4u : 28u;
+            x.m = 0;
+        } else {
+            // words hold no bits beyond their sites, so lo >> s leaves one
+            // nibble (p = 0) or clears the last one (p = 1)
+            x.s = p ? 4u : (uint32_t)sh_prev;
+            x.m = p ? 1u << sh_next : 16u;
+        }
+        return x;
+    }
+    __device__ __forceinline__ uint32_t xjoin(uint32_t lo, uint32_t hi, const XShift& x) const
+    {
+        return FAST ? __funnelshift_r(lo, hi, x.s) : (lo >> x.s) + hi * x.m;
     }
 
-    // Bulk row, 2 <= t < L_t, all links full beta.  up: offset of the t+1 row
-    // (rowW, or -(L_t - 1) rowW at t = L_t - 1); c0: Philox block of the word's
-    // first four sites.
-    __device__ __forceinline__ void bulk_item(uint32_t* own_b, const uint32_t* oth, int w, int up,
-                                              int p, uint32_t c0, uint32_t sweep, uint32_t c3) const
+    // What the two Philox blocks of every word of a half-sweep share: the rounds
+    // 0 and 1 up to the block index (counter word 0).
+    struct Stream {
+        uint32_t c3k, lo1k, h0k, l0;
+    };
+    __device__ __forceinline__ Stream stream(int c, uint32_t sweep) const
     {
-        const uint4 ua = philox_r0(c0, sweep, hi1, lo1, c3, K);
-        const uint4 ub = philox_r0(c0 + 1u, sweep, hi1, lo1, c3, K);
-        bulk_update(own_b, oth, w, up, p, ua, ub);
+        const uint64_t q0 = (uint64_t)kPhiloxM0 * (hi1 ^ sweep ^ K.k0[0]);
+        Stream x;
+        x.c3k = ((uint32_t)c | c3base) ^ K.k1[0];
+        x.lo1k = lo1 ^ K.k0[1];
+        x.h0k = (uint32_t)(q0 >> 32) ^ K.k1[1];
+        x.l0 = (uint32_t)q0;
+        return x;
     }
-
-    // The same update with the word's two Philox blocks (ua, ub) supplied.
-    __device__ __forceinline__ void bulk_update(uint32_t* own_b, const uint32_t* oth, int w, int up,
-                                                int p, const uint4& ua, const uint4& ub) const
+    // The block whose round 0 product is p0 = M0 * (block index).
+    __device__ __forceinline__ uint4 draw(uint64_t p0, const Stream& x) const
     {
-        const uint32_t own = ld(own_b, w, 1);
-        const uint32_t ntm = ld(oth, w - rowW(), 10);
-        const uint32_t ntp = ld(oth, w + up, 11);
-        const uint32_t nx0 = ld(oth, w, 5);
-        const uint32_t nx1 = xshift(oth, w, p, nx0);
-        uint32_t dsum = (own ^ ntm) + (own ^ ntp) + (own ^ nx0) + (own ^ nx1);
-        if (D == 3) dsum += (own ^ ld(oth, w + d_ym, 7)) + (own ^ ld(oth, w + d_yp, 8));
-        uint32_t flip = accept8<D>(dsum, ua, ub, tab);
-        if (!FAST) flip &= vmask;
-        st(own_b, w, own ^ flip, 9);
+        const uint64_t q1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ x.c3k);
+        return philox_from<2>((uint32_t)(q1 >> 32) ^ x.lo1k, (uint32_t)q1,
+                              x.h0k ^ (uint32_t)p0, x.l0, K);
     }
 
     // Site jl of a cut-row word that switches during the protocol: couplings
     // beta (1 - lambda) to its own replica (self_w), beta lambda to the next
-    // one (glue_w), tested against step k's table; replaces its flip bit.
-    // record: add its share of the work increment dE_k.
-    __device__ __forceinline__ void switched_site(uint32_t& flip, int jl, uint32_t own,
-                                                  uint32_t self_w, uint32_t glue_w, uint32_t dsum,
-                                                  const uint4& ua, const uint4& ub, int k,
-                                                  const TeamJob& J, int w_self, int w_glue,
-                                                  bool record, int& dE) const
+    // one (glue_w), tested against step k's table; returns its flip bit.  s:
+    // nibble-wise sums of its neighbours of spin -1, the self link's among them.
+    // With z = 4 (fixed links' sum) + 2 self + glue the table's index is z for
+    // a spin -1, 8D - 1 - z for a spin +1.  record: add its share of dE_k.
+    __device__ __forceinline__ uint32_t switched_site(int jl, uint32_t own, uint32_t self_w,
+                                                      uint32_t glue_w, uint32_t s, uint32_t u,
+                                                      const StepState& P, int& dE) const
     {
         const int sh = 4 * jl;
-        const uint32_t ob = (own >> sh) & 1u;
-        const int as = (int)(ob ^ ((self_w >> sh) & 1u));
-        const int ag = (int)(ob ^ ((glue_w >> sh) & 1u));
-        const int a_cnt = (int)((dsum >> sh) & 0xFu) - as;   // fixed links
-        const int a = (2 * D - 1) - 2 * a_cnt;
-        const int b = 1 - 2 * as;
-        const int cg = 1 - 2 * ag;
-        const int mm = a * J.den + b * w_self + cg * w_glue;
-        const int ti = (((a + 2 * D - 1) >> 1) * 2 + (b > 0)) * 2 + (cg > 0);
-        const bool acc = (mm <= 0) || (word8(ua, ub, jl) < __ldg(J.tcut + k * (8 * D) + ti));
-        flip = (flip & ~(0xFu << sh)) | ((uint32_t)acc << sh);
-        if (record) dE += b - cg;
+        const bool ob = (own >> sh) & 1u;
+        const int sf = (int)((self_w >> sh) & 1u), gl = (int)((glue_w >> sh) & 1u);
+        const int z = 4 * (int)((s >> sh) & 7u) - 2 * sf + gl;
+        const int ti = ob ? z : 8 * D - 1 - z;
+        const uint32_t T = __ldg(P.tk + ti);
+        // m <= 0 (always) is stored as 2^32 - 1, which a weakly coupled job's
+        // m > 0 can reach too
+        bool acc = u < T || T == 0xFFFFFFFFu;
+        if (J.weak && T == 0xFFFFFFFFu) {
+            const int a = 2 * (ti >> 2) - (2 * D - 1);
+            const int mm = a * J.den + ((ti & 2) ? P.w_self : -P.w_self) +
+                           ((ti & 1) ? P.w_glue : -P.w_glue);
+            acc = mm <= 0 || u != 0xFFFFFFFFu;
+        }
+        if (P.record) dE += ob ? 2 * (sf - gl) : 2 * (gl - sf);
+        return (uint32_t)acc << sh;
     }
 
-    // Row t of replica r (word w, row parity p), a row next to the cut (t = 0,
-    // 1) or a bulk row, in one instruction stream: a bulk row's neighbour
-    // "across" is its t+1 row with an empty glue mask, and only the switched
-    // sites of a cut row (k >= 0: the protocol step, whose table they use)
-    // take the per-site loop.  lg = columns glued across the cut.
-    __device__ __forceinline__ void row_update(uint32_t* own_b, const uint32_t* oth, int w, int t,
-                                               int r, int p, const uint4& ua, const uint4& ub,
-                                               int k, int lg, const TeamJob& J, int w_self,
-                                               int w_glue, bool record, int& dE) const
+    __device__ __forceinline__ Edge edge_of(int t) const
     {
-        const int Lt = g.Lt;
-        const int rw = rowW();
-        const int repW = Lt * rw;
-        const int n = g.nrep;
-        const bool cut = t < 2;
-        // the ordinary time neighbour (t - 1; t = 2 for the cut row t = 1)
-        const int off_n = t == 0 ? (Lt - 1) * rw : (t == 1 ? (Lt == 2 ? -rw : rw) : -rw);
-        // the row across the cut (t = 0, 1), else t + 1
-        const int off_x = t == 0 ? rw : t == 1 ? -rw : (t == Lt - 1 ? -(Lt - 1) * rw : rw);
-        // the glued partner across the cut: replica r+1 above it, r-1 below (mod n)
-        const int off_g = !cut ? 0 : t == 0 ? (r == n - 1 ? -(n - 1) * repW : repW)
-                                           : (r == 0 ? (n - 1) * repW : -repW);
-        const uint32_t m = cut ? glue_mask(lg, p) : 0u;
-        const uint32_t own = ld(own_b, w, 1);
-        const uint32_t nrm = ld(oth, w + off_n, 2);
-        const uint32_t self_w = ld(oth, w + off_x, 3);
-        const uint32_t glue_w = ld(oth, w + off_x + off_g, 4);
-        const uint32_t cross = (self_w & ~m) | (glue_w & m);
-        const uint32_t nx0 = ld(oth, w, 5);
-        const uint32_t nx1 = xshift(oth, w, p, nx0);
-        uint32_t dsum = (own ^ nrm) + (own ^ cross) + (own ^ nx0) + (own ^ nx1);
-        if (D == 3) dsum += (own ^ ld(oth, w + d_ym, 7)) + (own ^ ld(oth, w + d_yp, 8));
-        uint32_t flip = accept8<D>(dsum, ua, ub, tab);
-        // Switching sites g0 <= x < g1 during the protocol: couplings
-        // beta (1 - lambda) to their own replica, beta lambda to the next one.
-        // Site j of the word has x = 2 (8q + j) + p.
-        const int jlo = (cut && k >= 0) ? max(((J.g0 - p + 1) >> 1) - 8 * q, 0) : 8;
-        const int jhi = min(((J.g1 - p + 1) >> 1) - 8 * q, 8);
-#pragma unroll 1
-        for (int jl = jlo; jl < jhi; ++jl)
-            switched_site(flip, jl, own, self_w, glue_w, dsum, ua, ub, k, J, w_self, w_glue,
-                          record, dE);
-        if (!FAST) flip &= vmask;
-        st(own_b, w, own ^ flip, 9);
+        const int lt = Lt(), rw = 4 * rowW(), repW = lt * rw, n = g.nrep;
+        Edge e;
+        e.t = t;
+        e.n = t == 0 ? (lt - 1) * rw : (t == 1 ? (lt == 2 ? -rw : rw) : -rw);
+        e.x = t == 0 ? rw : t == 1 ? -rw : (t == lt - 1 ? -(lt - 1) * rw : rw);
+        e.g = t == 0 ? repW : t == 1 ? -repW : 0;
+        e.gw = t == 0 ? -(n - 1) * repW : t == 1 ? (n - 1) * repW : 0;
+        e.rw = t == 0 ? n - 1 : 0;
+        return e;
     }
 
-    __device__ __forceinline__ void half_sweep(int c, uint32_t sweep, int k, int lg,
-                                               const TeamJob& J, int w_self, int w_glue,
-                                               bool record, int& dE) const
+    // Bulk row, 2 <= t < L_t, all links full beta.  o: the word's position in
+    // the other colour; own: in its own; up: byte offset of the t+1 row.
+    __device__ __forceinline__ void bulk_row(A own_b, A oth, A own, A o, int up, const XShift& x,
+                                             const uint4& ua, const uint4& ub) const
     {
-        const int rw = rowW();
-        const int Lt = g.Lt;
-        const int cw = g.nrep * Lt * rw;
-        uint32_t* own_b = S + c * cw;
-        const uint32_t* oth = S + (1 - c) * cw;
-        const uint32_t c3 = (uint32_t)c | c3base;
-        const int stride = TS * rw;
-        const uint32_t cstride = (uint32_t)(TS * Ly() * g.G);   // Philox blocks per TS slices
-        const int pc = (c + y) & 1;
-        const int wrap_up = -(Lt - 1) * rw;
-        if (t0 >= Lt) return;   // a thread without sites
+        const uint32_t ow = ld(own_b, own, 1);
+        uint32_t s = ld(oth, o - 4 * rowW(), 10) + ld(oth, o + up, 11) + ld(oth, o, 5) +
+                     xjoin(ld(oth, o + x.a, 6), ld(oth, o + x.b, 6), x);
+        if (D == 3) s += ld(oth, o + d_ym, 7) + ld(oth, o + d_yp, 8);
+        uint32_t f = flips(s, ow, ua, ub);
+        if (!FAST) f &= vmask;
+        st(own_b, own, ow ^ f, 9);
+    }
+
+    // What the edge rows of a half-sweep share: row parity p, glue mask m
+    // (nibbles with x < lg, empty for a row away from the cut) and the word's
+    // first switched site jlo (x = 2 (8q + j) + p, g0 <= x < g1; 8 if none).
+    struct Cut {
+        uint32_t m;
+        int jlo, p;
+    };
+    __device__ __forceinline__ Cut cut_of(const Edge& e, int c, const StepState& P) const
+    {
+        Cut k;
+        k.p = (c + y + e.t) & 1;
+        const bool cut = e.t < 2;
+        k.m = cut ? glue_mask(P.lg, k.p) : 0u;
+        k.jlo = cut && P.k >= 0 ? max(((J.g0 - k.p + 1) >> 1) - 8 * q, 0) : 8;
+        return k;
+    }
+
+    // Edge row of replica r in one instruction stream for cut rows and others;
+    // only the switched sites of a cut row take the per-site loop.
+    __device__ __forceinline__ void edge_row(A own_b, A oth, int w4, const Edge& e, const Cut& k,
+                                             int r, const XShift& x, const uint4& ua,
+                                             const uint4& ub, const StepState& P, int& dE) const
+    {
+        const A o = oth + w4;
+        const uint32_t own = ld(own_b, own_b + w4, 1);
+        const uint32_t nrm = ld(oth, o + e.n, 2);
+        const uint32_t self_w = ld(oth, o + e.x, 3);
+        const uint32_t glue_w = ld(oth, o + e.x + (r == e.rw ? e.gw : e.g), 4);
+        const uint32_t cross = (self_w & ~k.m) | (glue_w & k.m);
+        uint32_t s = nrm + cross + ld(oth, o, 5) +
+                     xjoin(ld(oth, o + x.a, 6), ld(oth, o + x.b, 6), x);
+        if (D == 3) s += ld(oth, o + d_ym, 7) + ld(oth, o + d_yp, 8);
+        uint32_t f = flips(s, own, ua, ub);
+        if (k.jlo < 8) {
+            const int jhi = min(((J.g1 - k.p + 1) >> 1) - 8 * q, 8);
 #pragma unroll 1
-        for (int r = r0; r < g.nrep; r += RS) {
-            int t = t0;
-            int w = (r * Lt + t0) * rw + y * W() + q;
-            uint32_t c0 = (uint32_t)(((r * Lt + t0) * Ly() + y) * g.G + 2 * q);
-            // The thread's first row, cut (t0 < 2) or bulk, in one stream for
-            // the whole team; with TS = 1 the team's second row (t = 1) is a
-            // cut row too.  The rest are bulk rows.
-            do {
-                const uint4 ua = philox_r0(c0, sweep, hi1, lo1, c3, K);
-                const uint4 ub = philox_r0(c0 + 1u, sweep, hi1, lo1, c3, K);
-                row_update(own_b, oth, w, t, r, (pc ^ t) & 1, ua, ub, k, lg, J, w_self, w_glue,
-                           record, dE);
-                t += TS;
-                w += stride;
-                c0 += cstride;
-            } while (t < 2 && t < Lt);
-            if (TS & 1) {
-                for (; t < Lt; t += TS, w += stride, c0 += cstride)
-                    bulk_item(own_b, oth, w, t == Lt - 1 ? wrap_up : rw, (pc ^ t) & 1, c0, sweep,
-                              c3);
-            } else {
-                // t keeps its parity: the x-shift direction is fixed for the row set.
-                // Each row's update runs beside the Philox blocks of the next row
-                // (they do not depend on spins), so one warp's instruction stream
-                // mixes the wide multiplies with the update's logic; the blocks'
-                // round-0 products M0 c0 advance by additions.
-                const int p = (pc ^ t0) & 1;
-                if constexpr (CLT > 0 && CTS > 0 && CLT % CTS == 0 && CLT / CTS >= 3) {
-                    // L_t and the slice step fixed at compile time: the rows
-                    // t0 + k CTS, k = 1 .. L_t/CTS - 1, unrolled with immediate
-                    // word offsets (no loop or address arithmetic per row)
-                    constexpr int NROW = CLT / CTS;
-                    constexpr int STR = CTS * (D == 2 ? 1 : CLY) * CW;
-                    const int up_last = t0 == CTS - 1 ? wrap_up : rw;
-                    uint64_t p0 = (uint64_t)kPhiloxM0 * c0;
-                    const uint64_t dp = (uint64_t)kPhiloxM0 * cstride;
-                    uint4 ua = philox_p0(p0, sweep, hi1, lo1, c3, K);
-                    uint4 ub = philox_p0(p0 + kPhiloxM0, sweep, hi1, lo1, c3, K);
+            for (int jl = k.jlo; jl < jhi; ++jl)
+                f = (f & ~(0xFu << (4 * jl))) |
+                    switched_site(jl, own, self_w, glue_w, s, word8(ua, ub, jl), P, dE);
+        }
+        if (!FAST) f &= vmask;
+        st(own_b, own_b + w4, own ^ f, 9);
+    }
+
+    // A replica's bulk rows, from word w4 (byte offset) and Philox product p0 on.
+    // ODD: the slice step is odd, so the row parity alternates, starting with p.
+    template <bool ODD>
+    __device__ __forceinline__ void bulk_rows(A own_b, A oth, int w4, uint64_t p0, int p, XShift x,
+                                              const Stream& st) const
+    {
+        int n = n_bulk;
+        const uint64_t dp = (uint64_t)kPhiloxM0 * (uint32_t)(step() * Ly() * G());
+        const int stride = step() * rowW() * 4;
+        A own = own_b + w4, o = oth + w4;
+        auto row = [&](int up) {
+            const uint4 ua = draw(p0, st);
+            const uint4 ub = draw(p0 + kPhiloxM0, st);
+            bulk_row(own_b, oth, own, o, up, x, ua, ub);
+            p0 += dp;
+            own += stride;
+            o += stride;
+            if (ODD) x = xshift(p ^= 1);
+        };
+        int up = 4 * rowW();
+        if constexpr (CLT > 0 && CTS > 2 && CLT % CTS == 0) {
 #pragma unroll
-                    for (int k = 1; k < NROW - 1; ++k) {
-                        p0 += dp;
-                        const uint4 na = philox_p0(p0, sweep, hi1, lo1, c3, K);
-                        const uint4 nb = philox_p0(p0 + kPhiloxM0, sweep, hi1, lo1, c3, K);
-                        bulk_update(own_b, oth, w + (k - 1) * STR, rw, p, ua, ub);
-                        ua = na;
-                        ub = nb;
-                    }
-                    bulk_update(own_b, oth, w + (NROW - 2) * STR, up_last, p, ua, ub);
-                } else if (t < Lt) {
-                    uint64_t p0 = (uint64_t)kPhiloxM0 * c0;
-                    const uint64_t dp = (uint64_t)kPhiloxM0 * cstride;
-                    uint4 ua = philox_p0(p0, sweep, hi1, lo1, c3, K);
-                    uint4 ub = philox_p0(p0 + kPhiloxM0, sweep, hi1, lo1, c3, K);
-                    for (; t < Lt - TS; t += TS, w += stride, c0 += cstride) {
-                        p0 += dp;
-                        const uint4 na = philox_p0(p0, sweep, hi1, lo1, c3, K);
-                        const uint4 nb = philox_p0(p0 + kPhiloxM0, sweep, hi1, lo1, c3, K);
-                        bulk_update(own_b, oth, w, rw, p, ua, ub);
-                        ua = na;
-                        ub = nb;
-                    }
-                    bulk_update(own_b, oth, w, t == Lt - 1 ? wrap_up : rw, p, ua, ub);
-                }
+            for (int k = 1; k < CLT / CTS; ++k) row(up);
+        } else {
+            // four rows per pass; the last row, whose t + 1 row may wrap
+            // around, is one of the single rows that follow
+#pragma unroll 1
+            for (; n > 4; n -= 4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) row(up);
+            }
+#pragma unroll 1
+            for (; n > 0; --n) {
+                if (n == 1) up = up_last;
+                row(up);
             }
         }
     }
 
-    // Threads that own one row of each colour (a team with a thread per word
-    // of the lattice): the Philox blocks of half-sweep (sweep, c) of that row.
-    // They depend on the sweep index and the colour only, never on spins, so
-    // they can be drawn a half-sweep ahead.
-    __device__ __forceinline__ void row_draw(uint32_t sweep, int c, uint4& ua, uint4& ub) const
+    // The half-sweep of colour c.  With TS >= 3 slice steps slot t0 starts with
+    // row t0 - 1 (slot 0 with L_t - 1): the two rows next to the cut and the row
+    // whose t + 1 neighbour wraps around are all first rows, one instruction
+    // stream for the whole team, and every other row is t0 - 1 + k TS with plain
+    // time neighbours.  With TS <= 2 the cut rows t = 0, 1 come first and the
+    // last bulk row wraps.
+    __device__ __forceinline__ void half_sweep(int c, uint32_t sweep, const StepState& P,
+                                               int& dE) const
     {
-        const uint32_t c0 = (uint32_t)(((r0 * g.Lt + t0) * Ly() + y) * g.G + 2 * q);
-        const uint32_t c3 = (uint32_t)c | c3base;
-        ua = philox_r0(c0, sweep, hi1, lo1, c3, K);
-        ub = philox_r0(c0 + 1u, sweep, hi1, lo1, c3, K);
-    }
-
-    // The half-sweep of colour c over this thread's one row, blocks supplied.
-    __device__ __forceinline__ void row_half_sweep(int c, const uint4& ua, const uint4& ub, int k,
-                                                   int lg, const TeamJob& J, int w_self,
-                                                   int w_glue, bool record, int& dE) const
-    {
-        const int Lt = g.Lt;
-        if (t0 >= Lt) return;   // a thread without sites
         const int rw = rowW();
-        const int repW = Lt * rw;
-        const int n = g.nrep;
-        const int w = (r0 * Lt + t0) * rw + y * W() + q;
-        row_update(S + c * n * repW, S + (1 - c) * n * repW, w, t0, r0, (c + y + t0) & 1, ua, ub,
-                   k, lg, J, w_self, w_glue, record, dE);
+        const int lt = Lt();
+        const A own_b = colour(c), oth = colour(c ^ 1);
+        const int ts = step();
+        if (t0 >= lt) return;   // a thread without sites
+        const Stream st = stream(c, sweep);
+        const bool rot = ts >= 3;
+        const Cut k0 = cut_of(edge, c, P);
+        const XShift x0 = xshift(k0.p);
+#pragma unroll 1
+        for (int r = r0; r < g.nrep; r += RS) {
+            const int wr = r * lt * rw + y * W() + q;   // word of slice 0
+            const uint32_t cr = (uint32_t)((r * lt * Ly() + y) * G() + 2 * q);
+            auto first = [&](const Edge& e, const Cut& k, const XShift& x) {
+                const uint64_t p0 = (uint64_t)kPhiloxM0 * (cr + (uint32_t)(e.t * Ly() * G()));
+                const uint4 ua = draw(p0, st);
+                const uint4 ub = draw(p0 + kPhiloxM0, st);
+                edge_row(own_b, oth, 4 * (wr + e.t * rw), e, k, r, x, ua, ub, P, dE);
+            };
+            if (rot) {
+                first(edge, k0, x0);
+            } else {
+#pragma unroll 1
+                for (int t = t0; t < 2; t += ts) {
+                    const Edge e = edge_of(t);
+                    const Cut k = cut_of(e, c, P);
+                    first(e, k, xshift(k.p));
+                }
+            }
+            const uint64_t p0 = (uint64_t)kPhiloxM0 * (cr + (uint32_t)(tb * Ly() * G()));
+            const int w4 = 4 * (wr + tb * rw);
+            const int p = (c + y + tb) & 1;
+            if (CTS == 0 && (ts & 1)) bulk_rows<true>(own_b, oth, w4, p0, p, xshift(p), st);
+            else bulk_rows<false>(own_b, oth, w4, p0, p, rot ? x0 : xshift(p), st);
+        }
     }
 
     // Loads a stored configuration (int8 +-1, natural order [r][t][y][x]) into
@@ -379,9 +561,8 @@ struct Traj {
     __device__ __forceinline__ void import_spins(const int8_t* src) const
     {
         const int rw = rowW();
-        const int cw = g.nrep * g.Lt * rw;
         for (int c = 0; c < 2; ++c) {
-            uint32_t* base = S + c * cw;
+            const A base = colour(c);
             for (int r = r0; r < g.nrep; r += RS) {
                 int w = (r * g.Lt + t0) * rw + y * W() + q;
                 for (int t = t0; t < g.Lt; t += TS, w += TS * rw) {
@@ -392,7 +573,7 @@ struct Traj {
                         const int x = 2 * (8 * q + j) + p;
                         if (x < g.L && src[row0 + x] < 0) v |= 1u << (4 * j);
                     }
-                    st(base, w, v, 12);
+                    st(base, base + 4 * w, v, 12);
                 }
             }
         }
@@ -401,14 +582,16 @@ struct Traj {
     __device__ __forceinline__ void hot_start() const
     {
         const int rw = rowW();
-        const int cw = g.nrep * g.Lt * rw;
         const uint32_t cstride = (uint32_t)(TS * Ly() * g.G);
+#pragma unroll 1
         for (int c = 0; c < 2; ++c) {
-            uint32_t* base = S + c * cw;
+            const A base = colour(c);
             const uint32_t c3 = (uint32_t)c | c3base | (1u << 30);
+#pragma unroll 1
             for (int r = r0; r < g.nrep; r += RS) {
                 int w = (r * g.Lt + t0) * rw + y * W() + q;
                 uint32_t c0 = (uint32_t)(((r * g.Lt + t0) * Ly() + y) * g.G + 2 * q);
+#pragma unroll 1
                 for (int t = t0; t < g.Lt; t += TS, w += TS * rw, c0 += cstride) {
                     const uint4 ua = philox_r0(c0, 0u, hi1, lo1, c3, K);
                     const uint4 ub = philox_r0(c0 + 1u, 0u, hi1, lo1, c3, K);
@@ -416,7 +599,7 @@ struct Traj {
                                        ((ua.w >> 31) << 12) | ((ub.x >> 31) << 16) |
                                        ((ub.y >> 31) << 20) | ((ub.z >> 31) << 24) |
                                        ((ub.w >> 31) << 28);
-                    st(base, w, v & vmask, 12);
+                    st(base, base + 4 * w, v & vmask, 12);
                 }
             }
         }
@@ -430,76 +613,189 @@ struct WarpBarrier {
     __device__ __forceinline__ void operator()() const { __syncwarp(); }
 };
 
+// The protocol's course through a trajectory's sweeps: thermalisation sweeps
+// 0 .. n_therm - 1 at the start geometry (forward lambda = 0: x < g0 glued;
+// reverse lambda = 1: x < g1 glued), then sweep i of step k is sweep n_therm +
+// k n_sweep + i.  One loop runs both, so that the half-sweep's code exists once.
+template <int D>
+struct Course {
+    const TeamJob& J;
+    uint32_t s;      // global sweep index
+    int k, left;     // step, sweeps left in it
+    StepState P;
+
+    __device__ __forceinline__ explicit Course(const TeamJob& J_) : J(J_)
+    {
+        const bool resume = J.k_begin > 0 || J.start_in;
+        s = resume ? (uint32_t)J.n_therm + (uint32_t)J.k_begin * (uint32_t)J.n_sweep : 0u;
+        k = J.k_begin - 1;
+        left = resume ? 0 : J.n_therm;
+        P = StepState{-1, J.dir > 0 ? J.g0 : J.g1, 0, 0, J.tcut, false};
+    }
+    // The next sweep's state for row y; false after the last one.
+    __device__ __forceinline__ bool next(int y)
+    {
+        if (left == 0) {
+            if (++k >= J.k_end) return false;
+            left = J.n_sweep;
+            // protocol 2: only column y = k / den moves; the columns before it
+            // sit at the end geometry, the ones after it at the start geometry
+            const int ya = J.prot == 2 ? k / J.den : 0;
+            const int kp = k + 1 - ya * J.den;
+            P.w_self = J.dir > 0 ? J.den - kp : kp;
+            P.w_glue = J.dir > 0 ? kp : J.den - kp;
+            P.k = k;
+            P.lg = J.g0;
+            P.tk = J.tcut + (size_t)k * (8 * D);
+            P.record = true;
+            if (J.prot == 2 && y != ya) {
+                P.k = -1;
+                P.lg = (y < ya) == (J.dir > 0) ? J.g1 : J.g0;
+            }
+        }
+        --left;
+        return true;
+    }
+};
+
+// A trajectory whose team has a thread per word (2D, L = 16 and n L_t <= 32: one
+// warp or less).  So few warps share an SM that nothing hides a half-sweep's
+// latency but the warp itself, so each half-sweep draws the next one's
+// Philox blocks and counts their thresholds (neither depends on spins) beside
+// its own update, both colours' own words stay in registers, and everything of
+// rounds 0 to 2 that does not depend on the sweep is computed once.
+template <bool FAST, class Tr, class Bar>
+__device__ __forceinline__ int run_rows(const Tr& tr, const Geom& g, const PhiloxKeys& K,
+                                        const TeamJob& J, Bar bar)
+{
+    const int w = tr.r0 * g.Lt + tr.t0;   // one word per row
+    const bool here = tr.t0 < g.Lt;
+    const auto e = tr.edge_of(tr.t0);
+    const int off_g = e.x + (tr.r0 == e.rw ? e.gw : e.g);
+    const bool cut = here && tr.t0 < 2;
+    uint32_t own[2] = {0u, 0u};
+    // per colour and block: the counter entering round 2 but for its word 2,
+    // and M0 times its word 0
+    uint32_t c1[2][2], plo[2][2], phi[2][2], lop[2];
+    int jlo[2], jhi[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        if (here) own[c] = tr.ld(tr.colour(c), tr.colour(c) + 4 * w, 1);
+        const int p = (c + tr.t0) & 1;
+        jlo[c] = cut ? max((J.g0 - p + 1) >> 1, 0) : 8;
+        jhi[c] = min((J.g1 - p + 1) >> 1, 8);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint32_t)(w * g.G + b);
+            const uint64_t q1 = (uint64_t)kPhiloxM1 *
+                                ((uint32_t)(p0 >> 32) ^ ((uint32_t)c | tr.c3base) ^ K.k1[0]);
+            const uint64_t q0 =
+                (uint64_t)kPhiloxM0 * ((uint32_t)(q1 >> 32) ^ tr.lo1 ^ K.k0[1]);
+            c1[c][b] = (uint32_t)q1 ^ K.k0[2];
+            plo[c][b] = (uint32_t)q0;
+            phi[c][b] = (uint32_t)(q0 >> 32) ^ K.k1[2];
+            lop[b] = (uint32_t)p0 ^ K.k1[1];
+        }
+    }
+    auto draw = [&](uint32_t sweep, int c, uint4 u[2]) {
+        const uint64_t q0 = (uint64_t)kPhiloxM0 * (tr.hi1 ^ sweep ^ K.k0[0]);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const uint64_t q1 = (uint64_t)kPhiloxM1 * ((uint32_t)(q0 >> 32) ^ lop[b]);
+            u[b] = philox_from<3>((uint32_t)(q1 >> 32) ^ c1[c][b], (uint32_t)q1,
+                                  phi[c][b] ^ (uint32_t)q0, plo[c][b], K);
+        }
+    };
+    int dE = 0;
+    Course<2> C(J);
+    uint4 u[2];
+    draw(C.s, 0, u);
+    uint32_t n = count8<2>(u[0], u[1], J.tb);
+    uint32_t m[2];
+    int lg = -1;
+    auto half = [&](int c) {
+        const auto own_b = tr.colour(c), oth = tr.colour(c ^ 1), o = oth + 4 * w;
+        uint32_t f = 0, nrm = 0, self_w = 0, glue_w = 0;
+        if (here) {
+            nrm = tr.ld(oth, o + e.n, 2);
+            self_w = tr.ld(oth, o + e.x, 3);
+            glue_w = tr.ld(oth, o + off_g, 4);
+        }
+        uint4 v[2];
+        draw(c ? C.s + 1u : C.s, c ^ 1, v);
+        const uint32_t nn = count8<2>(v[0], v[1], J.tb);
+        const uint32_t ow = own[c], nx0 = own[c ^ 1];
+        const int p = (c + tr.t0) & 1;
+        const uint32_t s = nrm + ((self_w & ~m[c]) | (glue_w & m[c])) + nx0 +
+                           __funnelshift_r(nx0, nx0, p ? 4 : 28);
+        f = flips_of_counts<2>(s, ow, n);
+        if (C.P.k >= 0) {
+#pragma unroll 1
+            for (int jl = jlo[c]; jl < jhi[c]; ++jl)
+                f = (f & ~(0xFu << (4 * jl))) |
+                    tr.switched_site(jl, ow, self_w, glue_w, s, word8(u[0], u[1], jl), C.P, dE);
+        }
+        own[c] = ow ^ f;
+        if (here) tr.st(own_b, own_b + 4 * w, own[c], 9);
+        u[0] = v[0];
+        u[1] = v[1];
+        n = nn;
+        bar();
+    };
+#pragma unroll 1
+    while (C.next(0)) {
+        if (C.P.lg != lg) {
+            lg = C.P.lg;
+            m[0] = cut ? tr.glue_mask(lg, tr.t0 & 1) : 0u;
+            m[1] = cut ? tr.glue_mask(lg, (tr.t0 + 1) & 1) : 0u;
+        }
+        half(0);
+        C.P.record = false;
+        half(1);
+        ++C.s;
+    }
+    return dE;
+}
+
 // Runs one whole trajectory with the team's threads.  Every thread sharing the
 // barrier calls it with the same job (trip counts match across teams); tid < 0
 // marks a thread without sites.  Returns this thread's share of sum_k dE_k
 // (the caller applies the direction's sign and, in protocol 2, the factor L_y
 // that makes W = (beta/N) W_int).
 // sin: the stored state to start from when J.k_begin > 0 or J.start_in (else unused).
-// ROW: every thread owns one row of each colour (the team has a thread per
-// word); each half-sweep then draws the next one's Philox blocks beside its
-// own update, so the independent chains cover the latency of the
-// shared-memory loads and the barrier that a team this small (one warp per
-// trajectory, few warps per SM) has no other warps to hide.
-template <int D, bool FAST, int CW, int CLY, bool ROW = false, int CLT = 0, int CTS = 0, class Bar>
+// ROW: the team has a thread per word (run_rows).
+template <int D, bool FAST, bool PAIR, bool HBM, int CW, int CLY, bool ROW = false, int CLT = 0,
+          int CTS = 0, class Bar>
 __device__ __forceinline__ int run_trajectory(const Geom& g, const PhiloxKeys& K, const TeamJob& J,
-                                              long long traj, uint32_t* S_team,
-                                              const uint32_t* tab, int tid, int nthr, Bar bar,
+                                              long long traj, uint32_t* S_team, const uint2* tab,
+                                              int tid, int nthr, Bar bar,
                                               const int8_t* sin = nullptr)
 {
-    const Traj<D, FAST, CW, CLY, CLT, CTS> tr(g, S_team, tab, K, (uint32_t)traj,
-                                    ((uint32_t)(J.dir < 0) << 1) | ((uint32_t)J.l << 2), tid, nthr);
-    int dE = 0;
-    // the global sweep index: thermalisation sweeps 0 .. n_therm - 1, then
-    // protocol sweep i of step k is n_therm + k n_sweep + i
-    const bool resume = J.k_begin > 0 || J.start_in;
-    uint32_t s = resume ? (uint32_t)J.n_therm + (uint32_t)J.k_begin * (uint32_t)J.n_sweep : 0u;
-    uint4 ua, ub;   // ROW: the blocks of the coming half-sweep
-    if constexpr (ROW) tr.row_draw(s, 0, ua, ub);
-    auto half = [&](int c, int kk, int lg, int ws, int wg, bool rec) {
-        if constexpr (ROW) {
-            uint4 na, nb;
-            tr.row_draw(c ? s + 1u : s, c ^ 1, na, nb);
-            tr.row_half_sweep(c, ua, ub, kk, lg, J, ws, wg, rec, dE);
-            ua = na;
-            ub = nb;
-        } else {
-            tr.half_sweep(c, s, kk, lg, J, ws, wg, rec, dE);
-        }
-        bar();
-    };
-    if (resume) {
+    const Traj<D, FAST, PAIR, HBM, CW, CLY, CLT, CTS> tr(g, S_team, tab, J, K, (uint32_t)traj,
+                                                         tid, nthr);
+    if (J.k_begin > 0 || J.start_in) {
         if (tid >= 0) tr.import_spins(sin);
-        bar();
     } else {
         tr.hot_start();
-        bar();
-        // thermalisation at the start geometry: forward lambda = 0 (x < g0
-        // glued), reverse lambda = 1 (x < g1 glued)
-        const int lg_therm = J.dir > 0 ? J.g0 : J.g1;
-        for (int i = 0; i < J.n_therm; ++i, ++s) {
-            half(0, -1, lg_therm, 0, 0, false);
-            half(1, -1, lg_therm, 0, 0, false);
-        }
     }
-    for (int k = J.k_begin; k < J.k_end; ++k) {
-        // protocol 2: only column y = k / den moves; the columns before it sit
-        // at the end geometry, the ones after it at the start geometry
-        const int ya = k / J.den;
-        const int kp = k + 1 - ya * J.den;
-        const int w_self = J.dir > 0 ? J.den - kp : kp;
-        const int w_glue = J.dir > 0 ? kp : J.den - kp;
-        int kk = k, lg = J.g0;
-        if (J.prot == 2 && tr.y != ya) {
-            kk = -1;
-            lg = (tr.y < ya) == (J.dir > 0) ? J.g1 : J.g0;
+    bar();
+    if constexpr (ROW) {
+        return run_rows<FAST>(tr, g, K, J, bar);
+    } else {
+        int dE = 0;
+        Course<D> C(J);
+#pragma unroll 1
+        while (C.next(tr.y)) {
+#pragma unroll 1
+            for (int c = 0; c < 2; ++c) {
+                tr.half_sweep(c, C.s, C.P, dE);
+                bar();
+                C.P.record = false;
+            }
+            ++C.s;
         }
-        for (int i = 0; i < J.n_sweep; ++i, ++s) {
-            half(0, kk, lg, w_self, w_glue, i == 0);
-            half(1, kk, lg, w_self, w_glue, false);
-        }
+        return dE;
     }
-    return dE;
 }
 
 // Writes a team's final configuration as int8 +-1 in the order [r][t][y][x].
@@ -539,6 +835,9 @@ __device__ __forceinline__ TeamJob team_job(const JobDesc& J, int ly)
     t.g1 = __ldg(&J.g1);
     t.den = t.prot == 2 ? t.n_step / ly : t.n_step;
     t.tcut = J.tcut;
+    t.weak = __ldg(&J.weak) != 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) t.tb[a] = __ldg(&J.tb[a]);
     return t;
 }
 
