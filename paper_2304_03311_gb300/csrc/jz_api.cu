@@ -786,8 +786,10 @@ void ising_replica_free(ising_ctx* ctx)
     cudaSetDevice(ctx->device);
     cudaStreamSynchronize(ctx->stream);
     for (DevBuf* b : {&ctx->tcut, &ctx->jobs, &ctx->work, &ctx->spins, &ctx->est_in,
-                      &ctx->est_out, &ctx->lattice})
+                      &ctx->est_out, &ctx->lattice, &ctx->therm})
         if (b->ptr) cudaFree(b->ptr);
+    if (ctx->est_scratch) cudaFree(ctx->est_scratch);
+    if (ctx->h_est) cudaFreeHost(ctx->h_est);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     cudaEventDestroy(ctx->ev_k0);
     cudaEventDestroy(ctx->ev_k1);
@@ -1050,16 +1052,40 @@ int estimator_reduce(ising_ctx* ctx, const int64_t* work_int, int n_traj, double
             return rc;
         src = (const long long*)ctx->est_in.ptr;
     }
-    if ((rc = ensure(ctx, ctx->est_out, 4 * sizeof(double)))) return rc;
     const int B = n_jack_bins < n_traj ? n_jack_bins : n_traj;
-    if ((rc = cuda_err(jz::launch_estimator(src, n_traj, beta / (double)n_step, direction, B,
-                                            (double*)ctx->est_out.ptr, st))))
-        return rc;
+    // The grid's scratch (8 KB) and the pinned words its last CTA writes the
+    // estimate to are allocated on the first call and kept, not charged to the
+    // budget (the jobs' memory is what it bounds); without them the one-CTA
+    // kernel runs and its result is copied.
+    if (!ctx->est_scratch) {
+        if (cudaMalloc(&ctx->est_scratch, jz::kEstScratch) != cudaSuccess) {
+            ctx->est_scratch = nullptr;
+            cudaGetLastError();
+        } else if (cudaHostAlloc((void**)&ctx->h_est, 4 * sizeof(double), cudaHostAllocDefault) !=
+                       cudaSuccess ||
+                   cudaMemsetAsync(ctx->est_scratch, 0, jz::kEstScratch, st) != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(ctx->est_scratch);
+            ctx->est_scratch = nullptr;
+        }
+    }
+    const double scale = beta / (double)n_step;
     double h[3];
-    if ((rc = cuda_err(cudaMemcpyAsync(h, ctx->est_out.ptr, 3 * sizeof(double),
-                                       cudaMemcpyDeviceToHost, st))))
-        return rc;
-    if ((rc = cuda_err(cudaStreamSynchronize(st)))) return rc;
+    if (ctx->est_scratch) {
+        if ((rc = cuda_err(jz::launch_estimator_grid(src, n_traj, scale, direction, B,
+                                                     ctx->est_scratch, ctx->h_est, st))) ||
+            (rc = cuda_err(cudaStreamSynchronize(st))))
+            return rc;
+        std::memcpy(h, ctx->h_est, sizeof h);
+    } else {
+        if ((rc = ensure(ctx, ctx->est_out, 4 * sizeof(double)))) return rc;
+        if ((rc = cuda_err(jz::launch_estimator(src, n_traj, scale, direction, B,
+                                                (double*)ctx->est_out.ptr, st))) ||
+            (rc = cuda_err(cudaMemcpyAsync(h, ctx->est_out.ptr, sizeof h, cudaMemcpyDeviceToHost,
+                                           st))) ||
+            (rc = cuda_err(cudaStreamSynchronize(st))))
+            return rc;
+    }
     *log_ratio = h[0];
     *delta_S2 = h[1];
     *delta_S2_err = h[2];

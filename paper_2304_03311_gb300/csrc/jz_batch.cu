@@ -101,7 +101,7 @@ estimator_batch_kernel(const EstJob* __restrict__ jobs, double* __restrict__ out
 {
     __shared__ double s_max[kMaxJackBlocksB], s_sum[kMaxJackBlocksB];
     __shared__ int s_lo[kMaxJackBlocksB + 1];
-    __shared__ double s_theta[kMaxJackBlocksB + 1];
+    __shared__ double s_theta[kMaxJackBlocksB + 1], s_exp[2 * kMaxJackBlocksB];
     const EstJob E = jobs[blockIdx.x];
     const int B = E.n_blocks, n = E.n;
     const int size = n / B;
@@ -122,7 +122,7 @@ estimator_batch_kernel(const EstJob* __restrict__ jobs, double* __restrict__ out
         if (lane == 0) { s_max[b] = m; s_sum[b] = acc; }
     }
     __syncthreads();
-    estimator_finish(s_max, s_sum, s_lo, B, n, E.direction, s_theta, out + 3 * blockIdx.x);
+    estimator_finish(s_max, s_sum, s_lo, B, n, E.direction, s_theta, s_exp, out + 3 * blockIdx.x);
 }
 
 // ------------------------------------------------------------------ launchers --

@@ -163,43 +163,95 @@ __device__ __forceinline__ uint4 philox_r0(uint32_t c0, uint32_t c1, uint32_t hi
                           (uint32_t)p0, K);
 }
 
+// Sum of v over a warp, in every lane.
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    return v;
+}
+
 // The last stage of the FP64 estimator of one job (Appendix A, eq.
 // Jarzynski_theorem; blocked jackknife), given each jackknife block's maximum
 // m_b of -W_i and shifted sum s_b = sum_i e^{-W_i - m_b} (rows lo[b] ..
-// lo[b+1] - 1).  Thread b < B forms the estimate without block b, thread B
-// the full one, both as max-shifted log-sum-exps over the blocks; thread 0
-// then writes out[0] = ln <e^-W>, out[1] = Delta S, out[2] = the jackknife
-// error.  Every thread of the CTA calls it (it holds a barrier).
+// lo[b+1] - 1, B <= 64 blocks): the estimate without each block b and the full
+// one as max-shifted log-sum-exps over the blocks; thread 0 writes out[0] = ln
+// <e^-W>, out[1] = Delta S, out[2] = the jackknife error.  Every thread of the
+// CTA, at least kEstFinish of them, calls it (it holds barriers); s_exp: 2 B words
+// of shared memory.
+//
+// What bounds it: one CTA's chain of FP64 operations at GB300's FP64 rate (two
+// lanes per clock and SM).  The maximum without block b is the overall one
+// unless block b alone holds it, so only two sets of B exponentials exist; one
+// thread forms each, four (B <= 32) or two threads share an estimate's sum, its
+// two logarithms run in two lanes, and the maxima compare as integers.
+constexpr int kEstFinish = 160;
 __device__ __forceinline__ void estimator_finish(const double* s_max, const double* s_sum,
                                                  const int* s_lo, int B, int n, int direction,
-                                                 double* s_theta, double* out)
+                                                 double* s_theta, double* s_exp, double* out)
 {
-    const int t = (int)threadIdx.x;
-    if (t == B || (t < B && B >= 2)) {
-        const int skip = t < B ? t : -1;
-        const int count = t < B ? n - (s_lo[t + 1] - s_lo[t]) : n;
-        double M = -INFINITY;
-        for (int b = 0; b < B; ++b) if (b != skip) M = fmax(M, s_max[b]);
-        double tot = 0.0;
-        for (int b = 0; b < B; ++b) if (b != skip) tot += s_sum[b] * exp(s_max[b] - M);
-        s_theta[t] = M + log(tot) - log((double)count);
+    const int t = (int)threadIdx.x, lane = t & 31;
+    // every warp: the largest block maximum, its block, the largest of the rest
+    auto key = [](double v) {   // order-preserving
+        const long long k = __double_as_longlong(v);
+        return k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFLL);
+    };
+    const long long none = key(-INFINITY);
+    long long k1 = lane < B ? key(s_max[lane]) : none;
+    long long k2 = lane + 32 < B ? key(s_max[lane + 32]) : none;
+    int top = lane;
+    if (k2 > k1) {
+        const long long x = k1;
+        k1 = k2;
+        k2 = x;
+        top = lane + 32;
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const long long a1 = __shfl_xor_sync(0xFFFFFFFFu, k1, o);
+        const long long a2 = __shfl_xor_sync(0xFFFFFFFFu, k2, o);
+        const int at = __shfl_xor_sync(0xFFFFFFFFu, top, o);
+        const bool up = a1 > k1 || (a1 == k1 && at < top);
+        const long long lower = up ? k1 : a1;
+        k2 = lower > k2 ? lower : k2;
+        k2 = a2 > k2 ? a2 : k2;
+        k1 = up ? a1 : k1;
+        top = up ? at : top;
+    }
+    auto val = [](long long k) {
+        return __longlong_as_double(k ^ ((k >> 63) & 0x7FFFFFFFFFFFFFFFLL));
+    };
+    const double m1 = val(k1), m2 = val(k2);
+    if (t < B) s_exp[t] = exp(s_max[t] - m1);
+    if (t >= 64 && t - 64 < B) s_exp[B + t - 64] = t - 64 == top ? 0.0 : exp(s_max[t - 64] - m2);
     __syncthreads();
-    if (t != 0) return;
+    const int P = B <= 32 ? 4 : 2;
+    const int est = t / P, part = t - est * P;
+    double tot = 0.0;
+    if (est <= B) {
+        const double* e = est == top ? s_exp + B : s_exp;
+        for (int b = part; b < B; b += P)
+            if (b != est) tot += s_sum[b] * e[b];
+    }
+    for (int o = P / 2; o > 0; o >>= 1) tot += __shfl_xor_sync(0xFFFFFFFFu, tot, o);
+    // lane `part` 0 takes ln of the sum, 1 that of the row count
+    const int count = est < B ? n - (s_lo[est + 1] - s_lo[est]) : n;
+    const double ln = est <= B && part < 2 ? log(part ? (double)count : tot) : 0.0;
+    const double ln_count = __shfl_xor_sync(0xFFFFFFFFu, ln, 1);
+    if (est <= B && part == 0) s_theta[est] = (est == top ? m2 : m1) + ln - ln_count;
+    __syncthreads();
+    if (t >= 32) return;
     const double sign = direction > 0 ? -1.0 : 1.0;
     const double full = s_theta[B];
     double err = 0.0;
     if (B >= 2) {
-        double mean = 0.0;
-        for (int b = 0; b < B; ++b) mean += sign * s_theta[b];
-        mean /= B;
-        double ss = 0.0;
-        for (int b = 0; b < B; ++b) {
-            const double d = sign * s_theta[b] - mean;
-            ss += d * d;
-        }
-        err = sqrt((double)(B - 1) / B * ss);
+        const double a = lane < B ? sign * s_theta[lane] : 0.0;
+        const double b = lane + 32 < B ? sign * s_theta[lane + 32] : 0.0;
+        const double mean = warp_sum(a + b) / B;
+        const double da = lane < B ? a - mean : 0.0, db = lane + 32 < B ? b - mean : 0.0;
+        err = sqrt((double)(B - 1) / B * warp_sum(da * da + db * db));
     }
+    if (t != 0) return;
     out[0] = full;
     out[1] = sign * full;
     out[2] = err;

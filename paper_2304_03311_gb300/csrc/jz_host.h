@@ -34,6 +34,13 @@ bool traj_pairs(const Geom& g, int teams, bool hbm);
 cudaError_t traj_occupancy(int D, const Geom& g, const LaunchShape& sh, int* ctas_per_sm);
 cudaError_t launch_estimator(const long long* w_int, int n, double scale, int direction,
                              int n_blocks, double* out, cudaStream_t st);
+// The same over a grid of CTAs.  scratch: kEstScratch bytes of device memory,
+// its first word zero before the first call (each call leaves it zero); calls
+// that share it must not overlap.
+constexpr int kEstMaxCtas = 512;
+constexpr size_t kEstScratch = 64 + kEstMaxCtas * 16;
+cudaError_t launch_estimator_grid(const long long* w_int, int n, double scale, int direction,
+                                  int n_blocks, void* scratch, double* out, cudaStream_t st);
 size_t sw_smem_bytes(const Geom& g);
 // Threads of one Swendsen-Wang CTA (one trajectory) for dimension D.
 int sw_cta_threads(int D);
@@ -75,6 +82,8 @@ struct ising_ctx {
     size_t budget = 0;   // 0 = unlimited
     size_t used = 0;
     DevBuf tcut, jobs, work, spins, est_in, est_out;
+    void* est_scratch = nullptr;   // estimator_reduce's partial sums (kEstScratch bytes)
+    double* h_est = nullptr;       // and its result, in pinned memory
     DevBuf lattice;   // HBM lattices of shapes too large for shared memory
     DevBuf therm;     // spins after Swendsen-Wang thermalisation (therm_update = 1)
     std::vector<uint32_t> h_tcut;

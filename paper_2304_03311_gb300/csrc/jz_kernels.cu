@@ -2,6 +2,7 @@
 // trajectory kernel (jz_traj_kernel.cuh).
 #include <cstdint>
 
+#include "jz_host.h"
 #include "jz_traj_kernel.cuh"
 
 namespace jz {
@@ -12,6 +13,7 @@ namespace jz {
 // (Appendix A, eq. Jarzynski_theorem; blocked jackknife).
 // out[0] = ln <e^-W>, out[1] = Delta S_2, out[2] = jackknife error.
 constexpr int kMaxJackBlocks = 64;
+constexpr int kEstThreads = 160;
 
 __global__ void __launch_bounds__(1024)
 estimator_kernel(const long long* __restrict__ w_int, int n, double scale, int direction,
@@ -19,7 +21,7 @@ estimator_kernel(const long long* __restrict__ w_int, int n, double scale, int d
 {
     __shared__ double s_max[kMaxJackBlocks], s_sum[kMaxJackBlocks];
     __shared__ int s_lo[kMaxJackBlocks + 1];
-    __shared__ double s_theta[kMaxJackBlocks + 1];
+    __shared__ double s_theta[kMaxJackBlocks + 1], s_exp[2 * kMaxJackBlocks];
     const int B = n_blocks;
     const int size = n / B;
     if (threadIdx.x <= B) s_lo[threadIdx.x] = threadIdx.x == B ? n : threadIdx.x * size;
@@ -39,7 +41,85 @@ estimator_kernel(const long long* __restrict__ w_int, int n, double scale, int d
         if (lane == 0) { s_max[b] = m; s_sum[b] = acc; }
     }
     __syncthreads();
-    estimator_finish(s_max, s_sum, s_lo, B, n, direction, s_theta, out);
+    estimator_finish(s_max, s_sum, s_lo, B, n, direction, s_theta, s_exp, out);
+}
+
+// The same estimate by a grid of B x C CTAs: CTA (b, c) reduces chunk c of
+// jackknife block b to its maximum and shifted sum in part[], and the last
+// CTA to finish (counted in *done, which it sets back to 0) joins the chunks
+// and forms the estimates.
+//
+// What bounds it: FP64 exponentials, about 20 FP64 operations each, at two FP64
+// lanes per clock and SM: 16384 of them take one SM 85 us and 128 SMs under 1 us.
+// One value per thread where the SMs allow it.  16384 values, B = 32, whole
+// call: 153 us on one CTA -> 26 us on 128 (kernel about 15 us).
+__global__ void __launch_bounds__(kEstThreads)
+estimator_grid_kernel(const long long* __restrict__ w_int, int n, double scale, int direction,
+                      int B, int C, double2* part, unsigned int* done, double* __restrict__ out)
+{
+    __shared__ double s_max[kMaxJackBlocks], s_sum[kMaxJackBlocks];
+    __shared__ int s_lo[kMaxJackBlocks + 1];
+    __shared__ double s_theta[kMaxJackBlocks + 1], s_exp[2 * kMaxJackBlocks];
+    __shared__ double s_red[2][kEstThreads / 32], s_part[kEstMaxCtas];
+    __shared__ bool s_last;
+    const int t = (int)threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int size = n / B;
+    const int b = (int)blockIdx.x / C, c = (int)blockIdx.x - b * C;
+    const int len = b == B - 1 ? n - b * size : size;
+    const int lo = b * size + (int)((long long)len * c / C);
+    const int hi = b * size + (int)((long long)len * (c + 1) / C);
+    auto reduce = [&](double v, bool mx, double* red) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double x = __shfl_xor_sync(0xFFFFFFFFu, v, o);
+            v = mx ? fmax(v, x) : v + x;
+        }
+        if (lane == 0) red[warp] = v;
+        __syncthreads();
+        v = red[0];
+#pragma unroll
+        for (int i = 1; i < kEstThreads / 32; ++i) v = mx ? fmax(v, red[i]) : v + red[i];
+        return v;
+    };
+    const int i0 = lo + t;
+    const double x0 = i0 < hi ? -scale * (double)w_int[i0] : -INFINITY;
+    double m = x0;
+    for (int i = i0 + kEstThreads; i < hi; i += kEstThreads)
+        m = fmax(m, -scale * (double)w_int[i]);
+    m = reduce(m, true, s_red[0]);
+    double acc = i0 < hi ? exp(x0 - m) : 0.0;
+    for (int i = i0 + kEstThreads; i < hi; i += kEstThreads)
+        acc += exp(-scale * (double)w_int[i] - m);
+    acc = reduce(acc, false, s_red[1]);
+    if (t == 0) {
+        part[blockIdx.x] = make_double2(m, acc);
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (t <= B) s_lo[t] = t == B ? n : t * size;
+    if (t < B) {
+        double M = -INFINITY;
+        for (int k = 0; k < C; ++k) M = fmax(M, __ldcg(&part[t * C + k].x));
+        s_max[t] = M;
+    }
+    __syncthreads();
+    for (int i = t; i < B * C; i += kEstThreads) {
+        const double2 p = __ldcg(&part[i]);
+        const double M = s_max[i / C];
+        s_part[i] = p.x == M ? p.y : p.y * exp(p.x - M);
+    }
+    __syncthreads();
+    if (t < B) {
+        double S = 0.0;
+        for (int k = 0; k < C; ++k) S += s_part[t * C + k];
+        s_sum[t] = S;
+    }
+    if (t == 0) *done = 0u;
+    __syncthreads();
+    estimator_finish(s_max, s_sum, s_lo, B, n, direction, s_theta, s_exp, out);
 }
 
 // ------------------------------------------------------------ host launchers --
@@ -106,6 +186,19 @@ cudaError_t launch_estimator(const long long* w_int, int n, double scale, int di
                              int n_blocks, double* out, cudaStream_t st)
 {
     estimator_kernel<<<1, 1024, 0, st>>>(w_int, n, scale, direction, n_blocks, out);
+    return cudaGetLastError();
+}
+
+// Chunks per jackknife block: one value per thread up to kEstMaxCtas CTAs.
+cudaError_t launch_estimator_grid(const long long* w_int, int n, double scale, int direction,
+                                  int n_blocks, void* scratch, double* out, cudaStream_t st)
+{
+    int C = n / n_blocks / kEstThreads;
+    if (C > kEstMaxCtas / n_blocks) C = kEstMaxCtas / n_blocks;
+    if (C < 1) C = 1;
+    estimator_grid_kernel<<<n_blocks * C, kEstThreads, 0, st>>>(
+        w_int, n, scale, direction, n_blocks, C, (double2*)((char*)scratch + 64),
+        (unsigned int*)scratch, out);
     return cudaGetLastError();
 }
 
