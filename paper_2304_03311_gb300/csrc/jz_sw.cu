@@ -14,11 +14,16 @@
 //   B1 every site draws one Philox block (i, s, traj, dir<<1 | l<<2 | 2<<30);
 //      word w in {+x, +t same replica, +y, +t into replica r+1} activates that
 //      forward link when both spins are equal and the word is below the link's
-//      bond threshold floor(2^32 (1 - e^{-2K})).  +x bonds between lanes of
-//      one chunk form runs found by one ballot; each site's label is set to
-//      its run's first site.  The other active bonds become bits.  Block b
-//      of the flip stream (b, s, traj, dir<<1 | l<<2 | 3<<30) gives the flip
-//      bits of sites 128 b ... 128 b + 127 (words 0..3, bit i & 31).
+//      bond threshold floor(2^32 (1 - e^{-2K})).  +x bonds between sites of one
+//      32-site chunk and row form runs; each site's label is set to its run's
+//      first site.  The other active bonds become bits.  Block b of the flip
+//      stream (b, s, traj, dir<<1 | l<<2 | 3<<30) gives the flip bits of sites
+//      128 b ... 128 b + 127 (words 0..3, bit i & 31).  Two forms: `grouped`, a
+//      warp draws for up to 32 chunks, one lane per site, ballots turn the
+//      compares into words that lane k keeps for chunk k, and then a lane takes
+//      a chunk: the spins' equality is one word per direction, the spin bits
+//      shifted; and the plain form, a lane per site throughout, which small
+//      lattices (fewer than kGroupMin chunks per warp) take.
 //   B2 the recorded bonds, queued per warp and taken 32 at a time, merge
 //      clusters by lock-free union (the larger root is hooked under the
 //      smaller one, so the root of a cluster is its smallest site index);
@@ -30,9 +35,18 @@
 // not depend on the order of the unions, so the result is the same bit for bit
 // as a sequential union-find over the same bonds.
 //
+// What bounds it: issue (about 70 %) and the shared-memory latency of the walks.
+// Straight-line steps towards the root cost far less than a loop whose warp
+// follows its longest walk: with four of them ahead of every union and of every
+// root walk of the flip phase, unions that go on from the hooked root's old
+// parent instead of walking anew, and the grouped bond phase (156 -> 99
+// instructions per 32 sites and sweep), the 2D L = 64 scan of 31 x 64
+// trajectories takes 46 ms instead of 69 ms, 2D L = 128 23 ms (37), 3D 16^3 20 ms
+// (27), 3D 20^3 8.5 ms (13.3).
+//
 // Termination: a label always points to a site with a smaller or equal index
 // (equal only at a root), so every find walks a strictly decreasing chain (at
-// most V steps) and every retry of a union restarts from a strictly smaller
+// most V steps) and every retry of a union goes on from a strictly smaller
 // site.
 #include <cstdint>
 
@@ -46,15 +60,6 @@ namespace {
 // Threads per CTA (one trajectory): 256 in 2D, 512 in 3D, whose extra +y
 // bonds make the union phase longer (measured on 2D 64^2 and 3D 16^3).
 __host__ __device__ constexpr int sw_threads(int D) { return D == 3 ? 512 : 256; }
-
-// Minimum CTAs per SM for the register allocation.  0 for the shared-memory
-// variants leaves the choice to the compiler (40 registers; on the 2D L = 64
-// scan 7.5e10 site updates/s against 7.0e10 when sized for five CTAs, 48
-// registers); the HBM variants are sized so that they do not spill.
-__host__ __device__ constexpr int sw_min_ctas(int D, bool hbm)
-{
-    return hbm ? (D == 3 ? 3 : 5) : 0;
-}
 
 // Division by a fixed divisor d >= 1 for numerators n < 2^31 (Granlund and
 // Montgomery, PLDI'94): with s = ceil(log2 d) and m = floor(2^32 (2^s - d) / d)
@@ -84,7 +89,7 @@ struct SwGeom {
     int SL;       // sites of one time slice, L_y * L
     int VR;       // sites of one replica, L_t * SL
     int G;        // Philox blocks per colour row of the hot start, ceil(L / 8)
-    FastDiv dL, dLy, dLt;
+    FastDiv dL, dLy, dLt, dSL, dVR;
 };
 
 struct Site {
@@ -138,26 +143,88 @@ __device__ __forceinline__ int find_root(volatile int* lab, int a, int V)
     }
 }
 
+// Joins the clusters of a and b: up to four steps towards their roots, then the
+// larger node goes under the smaller one; what it pointed to before is joined in
+// turn.  A root that moved meanwhile costs one more step, not two new walks.
 __device__ __forceinline__ void merge(int* lab, int a, int b, int V)
 {
     volatile int* vl = lab;
-    for (;;) {
-        a = find_root(vl, a, V);
-        b = find_root(vl, b, V);
-        if (a == b) return;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        a = in_bounds(a, V, 21) ? vl[a] : 0;
+        b = in_bounds(b, V, 22) ? vl[b] : 0;
+    }
+    while (a != b) {
         if (a < b) {
             const int t = a;
             a = b;
             b = t;
         }
-        const int old = atomicMin(&lab[a], b);   // hook root a under b < a
+        const int old = atomicMin(&lab[a], b);
         if (old == a) return;
-        a = old;                                 // a was hooked meanwhile: retry from its parent
+        a = old;
     }
 }
 
-template <int D, bool HBM>
-__global__ void __launch_bounds__(sw_threads(D), sw_min_ctas(D, HBM))
+// The word of bits o .. o + 31 of a bit array with a readable word on each side.
+__device__ __forceinline__ uint32_t bits_at(const uint32_t* a, int o)
+{
+    const int w = o >> 5;
+    return __funnelshift_r(a[w], a[w + 1], (uint32_t)o & 31u);
+}
+
+__device__ __forceinline__ int mod(int a, const FastDiv& f)
+{
+    return a - (int)(fdiv((uint32_t)a, f) * f.d);
+}
+
+// Bits lo .. hi - 1 of a word, clipped to it.
+__device__ __forceinline__ uint32_t bit_range(int lo, int hi)
+{
+    lo = max(lo, 0);
+    hi = min(hi, 32);
+    if (lo >= hi) return 0u;
+    return (hi == 32 ? 0xFFFFFFFFu : (1u << hi) - 1u) & ~((1u << lo) - 1u);
+}
+
+// The bits of a word whose sites' residues (the first one's: r) lie in [lo, hi)
+// of a period.
+__device__ __forceinline__ uint32_t residue_bits(int r, int period, int lo, int hi)
+{
+    uint32_t m = 0;
+    for (int b = -r; b < 32; b += period) m |= bit_range(b + lo, b + hi);
+    return m;
+}
+
+// What the thread-per-word phases need of word q: residues of its first site
+// (in its row, replica, slice) and the bits of its sites at their row's end.
+struct WordPos {
+    int base, x, v, u;
+    uint32_t valid, E;
+};
+template <int D>
+__device__ __forceinline__ WordPos word_pos(const SwGeom& g, int q)
+{
+    WordPos p;
+    p.base = 32 * q;
+    p.x = mod(p.base, g.dL);
+    p.v = mod(p.base, g.dVR);
+    p.u = D == 3 ? mod(p.base, g.dSL) : p.x;
+    p.valid = bit_range(0, g.V - p.base);
+    p.E = residue_bits(p.x, g.L, g.L - 1, g.L);
+    return p;
+}
+
+// Words a warp draws for at once in the grouped bond phase: at most 32, the same
+// number of groups for every warp.
+__host__ __device__ __forceinline__ int sw_group(int VW, int n_warps)
+{
+    const int rounds = (VW + 32 * n_warps - 1) / (32 * n_warps);
+    return (VW + rounds * n_warps - 1) / (rounds * n_warps);
+}
+
+template <int D, bool HBM, bool GROUP, int MINB>
+__global__ void __launch_bounds__(sw_threads(D), MINB)
 sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, int n_jobs,
           uint32_t* __restrict__ gS, size_t g_words)
 {
@@ -223,6 +290,9 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
     }
     __syncthreads();
 
+    // B1: a warp draws for `group` words, then lane k takes the k-th one
+    const int group = sw_group(g.VW, n_warps);
+
     long long w = 0;
     const int sw_end = n_therm + k_end * n_sweep;
     for (int sw = k_begin > 0 ? n_therm + k_begin * n_sweep : 0; sw < sw_end; ++sw) {
@@ -269,10 +339,93 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
             if (4 * b + 2 < g.VW) fz[4 * b + 2] = u.z;
             if (4 * b + 3 < g.VW) fz[4 * b + 3] = u.w;
         }
-        // phase B1: bond draws.  A +x bond between two lanes of one warp
-        // chunk joins a run of consecutive sites; every site of a run gets the
-        // run's first site as its label (a star).  All other active bonds are
-        // recorded as bits for phase B2.
+        // phase B1: bond words.  Rounds 0 and 1 of a site's block are shared by
+        // the sweep up to the site index.
+        if constexpr (GROUP) {
+            const uint64_t q0 = (uint64_t)kPhiloxM0 * (hi1 ^ (uint32_t)sw ^ K.k0[0]);
+            const uint32_t h0k = (uint32_t)(q0 >> 32) ^ K.k1[1], l0 = (uint32_t)q0;
+            const uint32_t c3k = (c3 | (2u << 30)) ^ K.k1[0], lo1k = lo1 ^ K.k0[1];
+            for (int first = warp * group; first < g.VW; first += n_warps * group) {
+                uint32_t rx = 0, rt = 0, rg = 0, ry = 0;   // lane k: draws of word first + k
+                uint64_t pi = (uint64_t)kPhiloxM0 * (uint32_t)(32 * first + lane);
+                int v = mod(32 * first, g.dVR);            // the word's first site in its replica
+                const int count = min(group, g.VW - first);
+                for (int k = 0; k < count; ++k) {
+                    const uint64_t q1 = (uint64_t)kPhiloxM1 * ((uint32_t)(pi >> 32) ^ c3k);
+                    const uint4 d = philox_from<2>((uint32_t)(q1 >> 32) ^ lo1k, (uint32_t)q1,
+                                                   h0k ^ (uint32_t)pi, l0, K);
+                    pi += (uint64_t)kPhiloxM0 * 32u;
+                    uint32_t T_self = t_full, dg = 0;
+                    if (v < g.SL || v + 31 >= g.VR) {   // sites of slice t = 0
+                        uint32_t T_glue = 0;
+                        const int vi = mod(v + lane, g.dVR);
+                        if (vi < g.SL) {
+                            const int y = D == 3 ? (int)fdiv((uint32_t)vi, g.dL) : 0;
+                            const int x = D == 3 ? vi - y * g.L : vi;
+                            int side;   // of the link above this site: self, both, glued
+                            if (x >= g1) side = 0;
+                            else if (x < g0) side = 2;
+                            else if (ya >= 0 && y != ya) side = (y < ya) == (dir > 0) ? 2 : 0;
+                            else side = 1;
+                            if (side == 1) T_self = t_self;
+                            if (side == 2) T_self = 0u;
+                            T_glue = side == 1 ? t_glue : side == 2 ? t_full : 0u;
+                        }
+                        dg = __ballot_sync(0xFFFFFFFFu, d.w < T_glue);
+                    }
+                    const uint32_t dx = __ballot_sync(0xFFFFFFFFu, d.x < t_full);
+                    const uint32_t dt = __ballot_sync(0xFFFFFFFFu, d.y < T_self);
+                    const uint32_t dy = D == 3 ? __ballot_sync(0xFFFFFFFFu, d.z < t_full) : 0u;
+                    if (lane == k) {
+                        rx = dx;
+                        rt = dt;
+                        rg = dg;
+                        ry = dy;
+                    }
+                    v += 32;
+                    if (v >= g.VR) v = mod(v, g.dVR);
+                }
+                uint32_t m = 0;
+                if (lane < count) {
+                    const int q = first + lane;
+                    const WordPos p = word_pos<D>(g, q);
+                    const uint32_t W = sp[q];
+                    // bits of the sites equal to their neighbour at +o (wrapping: o - wrap)
+                    auto equal = [&](uint32_t wraps, int o, int wrap) {
+                        uint32_t nb = 0;
+                        if (~wraps & p.valid) nb = bits_at(sp, p.base + o) & ~wraps;
+                        if (wraps) nb |= bits_at(sp, p.base + o - wrap) & wraps;
+                        return ~(W ^ nb) & p.valid;
+                    };
+                    const uint32_t X = rx & equal(p.E & p.valid, 1, g.L);
+                    m = X & ~p.E & 0x7FFFFFFFu;
+                    bx[q] = X & ~m;
+                    const uint32_t A = residue_bits(p.v, g.VR, g.VR - g.SL, g.VR) & p.valid;
+                    bt[q] = rt & equal(A, g.SL, g.VR);
+                    if (D == 3) {
+                        const uint32_t B = residue_bits(p.u, g.SL, g.SL - g.L, g.SL) & p.valid;
+                        by[q] = ry & equal(B, g.L, g.SL);
+                    }
+                    uint32_t G = 0;
+                    rg &= p.valid;
+                    while (rg) {
+                        const int j = __ffs((int)rg) - 1, i = p.base + j;
+                        rg &= rg - 1u;
+                        const int r = (int)fdiv((uint32_t)i, g.dVR);
+                        if (spin_bit(sp, i + g.SL + glue_offset(g, r), g.V) ==
+                            (int)((W >> j) & 1u))
+                            G |= 1u << j;
+                    }
+                    bg[q] = G;
+                }
+                // every site's label is its run's first site
+                for (int k = 0; k < count; ++k) {
+                    const uint32_t brk = ~__shfl_sync(0xFFFFFFFFu, m, k) & ((1u << lane) - 1u);
+                    const int base = 32 * (first + k);
+                    if (base + lane < g.V) lab[base + lane] = base + 32 - __clz((int)brk);
+                }
+            }
+        } else {
         for (int base = warp * 32; base < g.V; base += chunk) {
             const int i = base + lane;
             bool ax = false, at = false, ay = false, ag = false, last = true;
@@ -330,6 +483,7 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
                 bg[q] = wg;
                 if (D == 3) by[q] = wy;
             }
+        }
         }
         __syncthreads();
         // phase B2: the recorded bonds merge clusters (+x bonds inside a
@@ -390,7 +544,21 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
             const int i = base + lane;
             int f = 0;
             if (i < g.V) {
-                const int root = find_root((volatile int*)lab, i, g.V);
+                volatile int* vl = lab;
+                int root = i;
+                if (GROUP) {
+#pragma unroll
+                    for (int h = 0; h < (HBM ? 3 : 4); ++h)
+                        root = in_bounds(root, g.V, 21) ? vl[root] : 0;
+                    for (;;) {
+                        const int up = in_bounds(root, g.V, 22) ? vl[root] : root;
+                        if (up == root) break;
+                        root = up;
+                    }
+                    vl[i] = root;
+                } else {
+                    root = find_root(vl, i, g.V);
+                }
                 f = (int)((fz[root >> 5] >> (root & 31)) & 1u);
             }
             const uint32_t m = __ballot_sync(0xFFFFFFFFu, f);
@@ -424,26 +592,54 @@ SwGeom make_swgeom(int D, const Geom& geo)
     g.dL = make_fastdiv((uint32_t)g.L);
     g.dLy = make_fastdiv((uint32_t)g.Ly);
     g.dLt = make_fastdiv((uint32_t)g.Lt);
+    g.dSL = make_fastdiv((uint32_t)g.SL);
+    g.dVR = make_fastdiv((uint32_t)g.VR);
     (void)D;
     return g;
 }
 
 }  // namespace
 
+using SwFn = void (*)(const SwGeom, const PhiloxKeys, const JobDesc*, int, uint32_t*, size_t);
+
+// group: the grouped bond phase, from kGroupMin words per warp on (states beyond
+// shared memory always).  n_cta <= 0: a full wave.
+//
+// Registers.  In shared memory the compiler's own choice (no occupancy asked
+// for) was the fastest: 2D L = 64 scan 48.8 ms, against 54.7, 54.2 and 56.3 ms when
+// sized for 4, 5 and 6 CTAs.  States beyond it wait on memory: as many CTAs as
+// fit (3 in 3D, 5 in 2D), but in 3D 64 registers without spills when two per SM
+// hold the whole launch anyway (L = 48, L_t = 192, 256 trajectories: 171 ms
+// against 190 ms; 456 trajectories of L = 40, L_t = 80: 68 ms against 49 ms).
+constexpr int kGroupMin = 6;
+static SwFn pick_sw(int D, bool hbm, bool group, long long n_cta)
+{
+    if (!hbm && D == 3)
+        return group ? sw_kernel<3, false, true, 0> : sw_kernel<3, false, false, 0>;
+    if (!hbm) return group ? sw_kernel<2, false, true, 0> : sw_kernel<2, false, false, 0>;
+    if (D == 2) return sw_kernel<2, true, true, 0>;
+    int dev = 0, n_sm = 0;
+    if (n_cta > 0 && cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        n_cta <= 2LL * n_sm)
+        return sw_kernel<3, true, true, 2>;
+    return sw_kernel<3, true, true, 3>;
+}
+
 int sw_cta_threads(int D) { return sw_threads(D); }
 
+// Their register counts (40 and 48) let 3 and 5 CTAs share an SM.  Not asked of
+// the runtime, which would load both kernels when a server starts.
 long long sw_hbm_wave(int D)
 {
-    int dev = 0, n_sm = 0, per_sm = 0;
-    auto kern = D == 3 ? sw_kernel<3, true> : sw_kernel<2, true>;
+    const int per_sm = D == 3 ? 3 : 5;
+    int dev = 0, n_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, sw_threads(D), 0) !=
-            cudaSuccess) {
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
         cudaGetLastError();
-        return sw_min_ctas(D, true);
+        return per_sm;
     }
-    return (long long)n_sm * (per_sm > 0 ? per_sm : 1);
+    return (long long)n_sm * per_sm;
 }
 
 cudaError_t bounds_status_sw(unsigned int out[2], bool clear)
@@ -477,8 +673,8 @@ cudaError_t launch_sw(int D, const Geom& geo, const PhiloxKeys& K, const JobDesc
     const SwGeom g = make_swgeom(D, geo);
     const size_t bytes = sw_smem_bytes(geo);
     const size_t smem = gS ? 0 : bytes;
-    auto kern = D == 3 ? (gS ? sw_kernel<3, true> : sw_kernel<3, false>)
-                       : (gS ? sw_kernel<2, true> : sw_kernel<2, false>);
+    const bool group = gS || sw_group(g.VW, sw_threads(D) / 32) >= kGroupMin;
+    const auto kern = pick_sw(D, gS != nullptr, group, n_cta);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
