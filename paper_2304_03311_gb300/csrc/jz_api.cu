@@ -294,17 +294,24 @@ jz::LaunchShape shape_for(const jz::Geom& g, int cta_threads)
 }
 
 // The relative rate of a launch of shape sh over n_traj trajectories of g
-// (n_traj <= 0: enough to fill every SM), fitted to rates measured on GB300
-// for every layout of 2D L = 34 .. 256 and 3D L = 8 .. 48 (L_t = L) at 256,
-// 2048 and 8192 trajectories:
-//   min(active warps per SM, kSatWarps) x (fraction of lanes owning a word)
-//   x R / (R + kBarrierRows) for one team per CTA,
-// where active warps are the resident ones (CUDA occupancy of the kernel
-// that runs g) or fewer when the trajectories do not fill the SMs, and R is
-// a thread's rows per half-sweep: a CTA team drains at its barrier, a warp
-// team's __syncwarp costs next to nothing.  Negative when sh cannot launch.
-constexpr double kSatWarps = 16.0;     // the integer pipes are saturated from here on
-constexpr double kBarrierRows = 1.5;   // a CTA barrier costs about 1.5 rows of work
+// (n_traj <= 0: enough to fill every SM): lattice words over the time of a
+// half-sweep, which for k CTAs resident on an SM is
+//   (sweep_cost + the CTA barrier) x (warps of the fullest SM sub-partition + kAlone).
+// The constants are fitted to rates measured on GB300 for every slice step of 2D L =
+// 64 .. 200 and 3D L = 8 .. 24 (L_t = L) at 256 and 4096 trajectories: per unit
+// of sweep_cost 3 warps per sub-partition take 0.78 of what 4 take; a barrier costs
+// little with other CTAs resident and about 8 units without; CTAs of five warps
+// three at a time run 4 % behind the model.  Up to kFewWaves waves the last wave,
+// CTAs that run with fewer others, counts by itself; in longer launches the CTAs
+// have drifted apart.  The busiest SM's CTAs decide: 256 trajectories on 152 SMs
+// last as long as two per SM.  Against the score before (active warps up to 16 per
+// SM x lanes owning a word x a barrier term), and with rows shared out by
+// split_rows: 2D L = 34 .. 240 and 3D L = 8 .. 36 run in 0.91 of the time on
+// average at 256 and 4096 trajectories (0.71 .. 1.03).  Negative when sh cannot
+// launch.
+constexpr double kAlone = 1.0;     // a sub-partition's fixed part, in warps
+constexpr double kBarrier = 4.0;   // a CTA barrier's cost beside other CTAs (sweep_cost's unit)
+constexpr int kFewWaves = 6;
 double shape_score(int d, const jz::Geom& g, const jz::LaunchShape& sh, long long n_traj,
                    int n_sm)
 {
@@ -317,31 +324,28 @@ double shape_score(int d, const jz::Geom& g, const jz::LaunchShape& sh, long lon
     }
     if (ctas < 1) return -1.0;
     const int wc = (sh.cta_threads + 31) / 32;
-    double warps = (double)ctas * wc;
-    if (n_traj > 0) {
-        const long long n_cta = (n_traj + sh.teams - 1) / sh.teams;
-        warps = std::min(warps, (double)n_cta * wc / n_sm);
-    }
-    const double lanes = (double)sh.teams * sh.team_threads / (32.0 * wc);
-    double sc = std::min(warps, kSatWarps) * lanes;
-    if (!sh.warp) {
-        const int ts = std::max(1, std::min(sh.team_threads / (g.GW * g.Ly), g.Lt));
-        const double rows = (double)g.nrep * g.Lt / ts;
-        sc *= rows / (rows + kBarrierRows);
-    }
-    return sc;
+    jz::RowKind kind;
+    const double cost = jz::sweep_cost(g, sh.team_threads, &kind);
+    const double words = (double)g.NR * g.GW * sh.teams;
+    auto time = [&](long long k) {   // of k resident CTAs
+        return (cost + (sh.warp ? 0.0 : kBarrier * (1.0 + 1.0 / k))) *
+               ((k * wc + 3) / 4 + kAlone + (wc == 5 && k > 1 ? 0.2 : 0.0));
+    };
+    const long long n_cta = (n_traj + sh.teams - 1) / sh.teams;
+    const long long m = (n_cta + n_sm - 1) / n_sm;   // CTAs of the busiest SM
+    if (n_traj <= 0 || m >= kFewWaves * ctas) return ctas * words / time(ctas);
+    const double t = (m / ctas) * time(ctas) + (m % ctas ? time(m % ctas) : 0.0);
+    return words * n_cta / n_sm / t;
 }
 
 // The shape a lattice in shared memory runs with when no CTA size is fixed.
 // Candidates: the warp-team layouts of shape_for for CTAs of 32 ... 512
 // threads, and one team per CTA for every slice step TS (col * TS <= 512).
 // shape_for(g, 0) is kept unless another candidate scores kKeepMargin more
-// (shape_score).  On the measured layouts this picks within about 2 % of the
-// fastest one on average and runs 1.39x the rate of shape_for(g, 0): narrow
-// slices of large lattices (2D L ~ 130 .. 240 with L_t = L), whose warp
-// teams each hold a whole lattice of shared memory and leave an SM four
-// warps, gain 1.4 - 1.9x as CTA teams; small jobs, whose trajectories fill
-// more SMs when each has more threads, 2 - 3x.  Lattices in HBM keep
+// (shape_score): narrow slices of large lattices (2D L ~ 130 .. 240 with L_t =
+// L), whose warp teams each hold a whole lattice of shared memory and leave an
+// SM four warps, gain 1.4 - 1.9x as CTA teams; small jobs, whose trajectories
+// fill more SMs when each has more threads, 2 - 3x.  Lattices in HBM keep
 // shape_for(g, 0).
 constexpr double kKeepMargin = 1.05;
 jz::LaunchShape default_shape(int d, const jz::Geom& g, long long n_traj)
@@ -1297,11 +1301,11 @@ cudaError_t launch_estimator_batch(const EstJob* jobs, int n_jobs, double* out, 
 }  // namespace jz
 
 // A job's layout inside the plan's CTAs of cta threads: the warp teams of
-// shape_for, or one team of the whole CTA when that keeps more of the CTA's
-// lanes busy (shape_score's barrier term).  A large lattice leaves most warps
-// of a warp-team CTA idle -- 2D L = 128 fits seven 32 KB lattices in a
-// 384-thread CTA -- and its shared memory would then set every CTA's, one
-// CTA per SM; as one team it holds one lattice.
+// shape_for, or one team of the whole CTA when that takes less of the CTA's time
+// per trajectory (sweep_cost).  A large lattice leaves most warps of a warp-team
+// CTA idle -- 2D L = 128 fits seven 32 KB lattices in a 384-thread CTA -- and
+// its shared memory would then set every CTA's, one CTA per SM; as one team it
+// holds one lattice.
 jz::LaunchShape plan_shape(const jz::Geom& g, int cta)
 {
     const jz::LaunchShape w = shape_for(g, cta);
@@ -1309,12 +1313,9 @@ jz::LaunchShape plan_shape(const jz::Geom& g, int cta)
     const int ts = std::min(cta / col, g.Lt);
     if (ts < 1 || col * ts < 32) return w;
     auto busy = [&](const jz::LaunchShape& sh) {
-        double b = (double)sh.teams * sh.team_threads / cta;
-        if (!sh.warp) {
-            const double rows = (double)g.nrep * g.Lt / std::min(sh.team_threads / col, g.Lt);
-            b *= rows / (rows + kBarrierRows);
-        }
-        return b;
+        jz::RowKind kind;
+        return sh.teams /
+               (jz::sweep_cost(g, sh.team_threads, &kind) + (sh.warp ? 0.0 : 2 * kBarrier));
     };
     jz::LaunchShape c{};
     c.team_threads = col * ts;
@@ -1453,8 +1454,8 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
         jz::BatchJob& B = bj[j];
         B.g = make_geom(p.d, p.L, p.L_t, nrep_of(p));
         B.D = p.d;
-        B.fast = (B.g.Lh % 8) == 0;   // rows of whole 8-site words
         B.sh = plan_shape(B.g, cta);
+        B.kind = jz::row_kind(B.g, B.sh);
         B.lattice_words = 2 * B.g.NR * B.g.GW;
         if (!shape_fits(B.g) || B.sh.team_threads > cta || (B.sh.warp && B.sh.cta_threads > cta)) {
             plan_release(pl);

@@ -17,7 +17,7 @@ namespace jz {
 
 constexpr int kMaxTeams = 64;
 
-template <int D, bool FAST, bool PAIR, class Bar>
+template <int D, int KIND, bool PAIR, class Bar>
 __device__ __forceinline__ void run_item(const BatchJob& B, const PhiloxKeys& K, int traj_lo,
                                          uint32_t* S, const uint2* tab, int* s_work, Bar bar)
 {
@@ -34,7 +34,7 @@ __device__ __forceinline__ void run_item(const BatchJob& B, const PhiloxKeys& K,
     const long long V = (long long)B.g.nrep * B.g.Lt * B.g.Ly * B.g.L;
     // therm_update = 1: the job starts from its thermalised spins
     const int8_t* sin = (has && tj.start_in) ? B.J.spins_in + local * V : nullptr;
-    const int dE = run_trajectory<D, FAST, PAIR, false, 0, 0>(B.g, K, tj, B.J.traj0 + local, St, tab, tid,
+    const int dE = run_trajectory<D, KIND, PAIR, false, 0, 0>(B.g, K, tj, B.J.traj0 + local, St, tab, tid,
                                                  B.sh.team_threads, bar, sin);
     if (has && dE != 0) atomicAdd(&s_work[tm], dE);
     __syncthreads();
@@ -47,12 +47,12 @@ __device__ __forceinline__ void run_item(const BatchJob& B, const PhiloxKeys& K,
                         tid, B.sh.team_threads);
 }
 
-template <int D, bool FAST, bool PAIR>
+template <int D, int KIND, bool PAIR>
 __device__ __forceinline__ void run_item_any(const BatchJob& B, const PhiloxKeys& K, int traj_lo,
                                              uint32_t* S, const uint2* tab, int* s_work)
 {
-    if (B.sh.warp) run_item<D, FAST, PAIR>(B, K, traj_lo, S, tab, s_work, WarpBarrier{});
-    else run_item<D, FAST, PAIR>(B, K, traj_lo, S, tab, s_work, CtaBarrier{});
+    if (B.sh.warp) run_item<D, KIND, PAIR>(B, K, traj_lo, S, tab, s_work, WarpBarrier{});
+    else run_item<D, KIND, PAIR>(B, K, traj_lo, S, tab, s_work, CtaBarrier{});
 }
 
 template <bool PAIR>
@@ -79,11 +79,15 @@ persistent_kernel(const BatchJob* __restrict__ jobs, const int2* __restrict__ it
         for (int i = threadIdx.x; i < kMaxTeams; i += blockDim.x) s_work[i] = 0;
         __syncthreads();
         if (B.D == 2) {
-            if (B.fast) run_item_any<2, true, PAIR>(B, K, item.y, S, s_tab, s_work);
-            else run_item_any<2, false, PAIR>(B, K, item.y, S, s_tab, s_work);
+            if (B.kind == kWhole) run_item_any<2, kWhole, PAIR>(B, K, item.y, S, s_tab, s_work);
+            else if (B.kind == kRagged)
+                run_item_any<2, kRagged, PAIR>(B, K, item.y, S, s_tab, s_work);
+            else run_item_any<2, kHalfTail, PAIR>(B, K, item.y, S, s_tab, s_work);
         } else {
-            if (B.fast) run_item_any<3, true, PAIR>(B, K, item.y, S, s_tab, s_work);
-            else run_item_any<3, false, PAIR>(B, K, item.y, S, s_tab, s_work);
+            if (B.kind == kWhole) run_item_any<3, kWhole, PAIR>(B, K, item.y, S, s_tab, s_work);
+            else if (B.kind == kRagged)
+                run_item_any<3, kRagged, PAIR>(B, K, item.y, S, s_tab, s_work);
+            else run_item_any<3, kHalfTail, PAIR>(B, K, item.y, S, s_tab, s_work);
         }
         __syncthreads();   // shared memory and s_item are reused by the next item
     }

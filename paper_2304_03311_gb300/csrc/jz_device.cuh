@@ -76,6 +76,59 @@ struct LaunchShape {
     int warp;
 };
 
+// How a team's slots (threads per word column) share the n L_t rows: TS slices
+// at a time in RS replicas at a time, and the half-sweep's length that follows,
+// in twelfths of a bulk row's time.
+struct RowSplit {
+    int ts, rs, cost;
+};
+
+// word: a bulk row's twelfths, 12 for a whole word, 7 for a half one.  A
+// thread's first row in each replica costs 8 more (the glued link and the cut
+// columns), so splitting the replicas (RS > 1) saves edge rows; it needs TS
+// >= 3, where one edge row per replica suffices.  With a whole time column per
+// slot (TS = L_t) the rest of the slots are replicas.
+__host__ __device__ inline RowSplit split_rows(int slots, int nrep, int Lt, int word)
+{
+    if (slots >= Lt) {
+        const int rs = slots / Lt;
+        return RowSplit{Lt, rs, ((nrep + rs - 1) / rs) * (word + 8)};
+    }
+    RowSplit b{slots, 1, nrep * (word * ((Lt + slots - 1) / slots) + (slots == 1 ? 16 : 8))};
+    for (int rs = 2; rs <= nrep && slots / rs >= 3; ++rs) {
+        const int ts = slots / rs;
+        const int cost = ((nrep + rs - 1) / rs) * (word * ((Lt + ts - 1) / ts) + 8);
+        if (cost < b.cost) b = RowSplit{ts, rs, cost};
+    }
+    return b;
+}
+
+// How a team works on a row's words: all alike, whole ones (kWhole) or the last
+// one ragged (kRagged); or, when the last word has at most four sites and needs
+// one Philox block only, these half words apart from the others (kHalfTail).
+enum RowKind { kRagged = 0, kWhole = 1, kHalfTail = 2 };
+
+// A half-sweep's length with a team of nthr threads (split_rows' unit), and the
+// kind it takes: half words apart where that is shorter.
+__host__ __device__ inline int sweep_cost(const Geom& g, int nthr, RowKind* kind)
+{
+    const int all = split_rows(nthr / (g.GW * g.Ly), g.nrep, g.Lt, 12).cost;
+    *kind = g.Lh % 8 == 0 ? kWhole : kRagged;
+    if (g.Lh % 8 == 0 || g.Lh % 8 > 4) return all;
+    const int whole =
+        g.GW == 1 ? 0 : split_rows(nthr / ((g.GW - 1) * g.Ly), g.nrep, g.Lt, 12).cost;
+    const int apart = whole + split_rows(nthr / g.Ly, g.nrep, g.Lt, 7).cost;
+    if (apart >= all) return all;
+    *kind = kHalfTail;
+    return apart;
+}
+__host__ __device__ inline RowKind row_kind(const Geom& g, const LaunchShape& sh)
+{
+    RowKind k;
+    sweep_cost(g, sh.team_threads, &k);
+    return k;
+}
+
 // Per-job (one transformation) parameters, device copy.
 struct JobDesc {
     int l;              // switched column
@@ -102,7 +155,7 @@ struct JobDesc {
 struct BatchJob {
     JobDesc J;            // thresholds, outputs, trajectory range
     Geom g;
-    int D, fast;
+    int D, kind;          // RowKind
     LaunchShape sh;       // team size, teams per CTA (= trajectories per work item), barrier
     int lattice_words;    // 2 * NR * GW spin words per team
 };

@@ -14,15 +14,20 @@
 // Nibble-wise sums of the neighbours' words give the number of neighbours of
 // spin -1 of all eight sites at once (at most 6, so no carries cross nibbles).
 //
-// Team mapping: a team of GW * L_y * TS * RS threads; thread (r0, t0, y, q)
-// owns word q of row y of every TS-th time slice in the replicas r0, r0 + RS,
-// ... and both colours, so all its index and wrap arithmetic is fixed.  RS > 1
-// only when TS = L_t (a whole time column per thread slot): lattices so small
-// that one replica's words leave most of a warp idle.  A replica's rows are one
-// or two edge rows, which blend in the glued replica and handle the switched
-// columns (half_sweep says which rows), and bulk rows.  CW, CLY > 0 fix GW and
-// L_y at compile time (neighbour loads then use immediate offsets); 0 reads
-// them from Geom.
+// Team mapping: the team's threads per word column are TS x RS slots; thread
+// (r0, t0, y, q) owns word q of row y of every TS-th time slice in the replicas
+// r0, r0 + RS, ... and both colours, so all its index and wrap arithmetic is
+// fixed.  split_rows chooses TS and RS for the shortest half-sweep.  A replica's
+// rows are one or two edge rows per thread, which blend in the glued replica and
+// handle the switched columns (half_sweep says which rows), and bulk rows; an
+// edge row costs about 90 instructions more, so two replicas on two sets of
+// slots, one edge row per thread, beat one set that has two (2D L = 128, L_t =
+// 1024 CTA teams: 109.7 -> 106.8 ms per 8-column scan).  Where the last word of
+// a row holds at most four sites, i.e. draws one Philox block, and it pays
+// (sweep_cost), these half words are shared out apart from the whole ones, and
+// no thread draws a block that no site uses (3D L = 24, L_t = 96: 121.4 -> 103.0
+// ms).  CW, CLY > 0 fix GW and L_y at compile time (neighbour loads then use
+// immediate offsets); 0 reads them from Geom.
 //
 // What bounds it (ncu and instruction-mix probes on GB300, cycles per SM
 // sub-partition and spin word of 32 lanes): the pipes that issue the two
@@ -74,23 +79,26 @@ __device__ __forceinline__ void add_if_lt(uint32_t& f, uint32_t u, uint32_t t)
         : "r"(u), "r"(t), "n"((int)(1u << SH)));
 }
 
-// PAIR acceptance, the form of every job that allows it: a 256-entry table of threshold pairs in shared memory,
-// indexed by one byte of v, i.e. by two sites at once.  Nibble j of v is site
+// PAIR acceptance, the form of every job that allows it: a 256-entry table of
+// threshold pairs in shared memory, indexed by one byte of v, i.e. by two sites at once.  Nibble j of v is site
 // j's state: its neighbours of spin -1 counted (at most 2D < 8), its own spin in
 // bit 3.  A site flips iff its draw is at most its threshold.  Returns the flip
-// bits (bit 4j); sites 0..3 use the words of block ua, sites 4..7 those of ub.
+// bits (bit 4j); sites 0..3 use the words of block ua, sites 4..7 those of ub (HALF:
+// a word of at most four sites).
+template <bool HALF>
 __device__ __forceinline__ uint32_t accept_pairs(uint32_t v, const uint4& ua, const uint4& ub,
                                                  const uint2* tab)
 {
     const uint2 t01 = tab[v & 0xFFu];
     const uint2 t23 = tab[__byte_perm(v, 0, 0x4441)];
-    const uint2 t45 = tab[__byte_perm(v, 0, 0x4442)];
-    const uint2 t67 = tab[v >> 24];
     uint32_t f = 0;
     add_if_le<0>(f, ua.x, t01.x);
     add_if_le<4>(f, ua.y, t01.y);
     add_if_le<8>(f, ua.z, t23.x);
     add_if_le<12>(f, ua.w, t23.y);
+    if (HALF) return f;
+    const uint2 t45 = tab[__byte_perm(v, 0, 0x4442)];
+    const uint2 t67 = tab[v >> 24];
     add_if_le<16>(f, ub.x, t45.x);
     add_if_le<20>(f, ub.y, t45.y);
     add_if_le<24>(f, ub.z, t67.x);
@@ -120,7 +128,7 @@ __device__ __forceinline__ void fill_pairs(uint2* tab, const uint32_t* __restric
 // table's 3.5 (3D: 6).  Nibble j of the result is the number of thresholds T[i],
 // i < D, above site j's draw.  tb grows with a, so the site flips iff
 // a + count >= D.  It depends on the draws alone.
-template <int D>
+template <int D, bool HALF = false>
 __device__ __forceinline__ uint32_t count8(const uint4& ua, const uint4& ub, const uint32_t* T)
 {
     uint32_t n = 0;
@@ -130,6 +138,7 @@ __device__ __forceinline__ uint32_t count8(const uint4& ua, const uint4& ub, con
         add_if_lt<4>(n, ua.y, T[i]);
         add_if_lt<8>(n, ua.z, T[i]);
         add_if_lt<12>(n, ua.w, T[i]);
+        if (HALF) continue;
         add_if_lt<16>(n, ub.x, T[i]);
         add_if_lt<20>(n, ub.y, T[i]);
         add_if_lt<24>(n, ub.z, T[i]);
@@ -153,6 +162,10 @@ __device__ __forceinline__ uint32_t word8(const uint4& ua, const uint4& ub, int 
 {
     return word_of(j < 4 ? ua : ub, j & 3);
 }
+
+// The words of a row that a thread set owns: all of them, or, where rows end in
+// half a word, the whole words and the half words apart.
+enum RowPart { kAllWords = 0, kWholeWords = 1, kTailWords = 2 };
 
 // Per-job values a team needs (read from the job descriptor once).
 struct TeamJob {
@@ -208,8 +221,10 @@ struct Mem<true> {
 
 // CLT, CTS > 0: L_t and the slice step TS fixed at compile time (the 2D L = 64,
 // L_t = 64 warp teams); 0 reads them from Geom and the team size.
-template <int D, bool FAST, bool PAIR, bool HBM, int CW = 0, int CLY = 0, int CLT = 0, int CTS = 0>
+template <int D, bool FAST, bool PAIR, bool HBM, int CW = 0, int CLY = 0, int CLT = 0, int CTS = 0,
+          int PART = kAllWords>
 struct Traj {
+    static constexpr bool HALF = PART == kTailWords;
     using M = Mem<HBM>;
     using A = typename M::A;
     // A thread's edge row (t = 0, 1 next to the cut, or any other, whose
@@ -234,13 +249,20 @@ struct Traj {
     int d_qm, d_qp;           // byte offset of the x-shift neighbour word (p = 0 / 1)
     int d_ym, d_yp;           // byte offsets of the rows y-1 / y+1 (3D)
     Edge edge;                // TS >= 3: the first row of each replica
-    int tb, n_bulk, up_last;  // first bulk row, their number, the last one's t + 1 row
+    int tb, n_all, up_last;   // first bulk row, the rows all slots have, the last one's t + 1 row
+    bool has_last;            // one row more
     uint32_t vmask;           // nibbles of word q that hold sites (ragged rows)
     int sh_next, sh_prev;     // ragged rows: nibble position of the wrapped x neighbour
 
     __device__ __forceinline__ int W() const { return CW > 0 ? CW : g.GW; }
     __device__ __forceinline__ int Ly() const { return D == 2 ? 1 : (CLY > 0 ? CLY : g.Ly); }
     __device__ __forceinline__ int rowW() const { return Ly() * W(); }
+    // words of a row that this thread set owns, from word first() on
+    __device__ __forceinline__ int own_words() const
+    {
+        return PART == kAllWords ? W() : PART == kWholeWords ? W() - 1 : 1;
+    }
+    __device__ __forceinline__ int first() const { return HALF ? W() - 1 : 0; }
     __device__ __forceinline__ int Lt() const { return CLT > 0 ? CLT : g.Lt; }
     // Philox blocks per row: full words have two each
     __device__ __forceinline__ int G() const { return CW > 0 && FAST ? 2 * CW : g.G; }
@@ -269,17 +291,20 @@ struct Traj {
         const uint64_t p1 = (uint64_t)kPhiloxM1 * traj;
         hi1 = (uint32_t)(p1 >> 32);
         lo1 = (uint32_t)p1;
-        const int col = W() * Ly();
+        const int wp = own_words();
+        if (wp == 0) tid = -1;   // rows of half a word have no whole one
+        const int col = max(wp, 1) * Ly();
         const int slots = nthr / col;   // threads per word column
-        TS = CTS > 0 ? CTS : (slots < g.Lt ? slots : g.Lt);
-        RS = slots / TS;
+        const RowSplit sp = split_rows(slots, g.nrep, g.Lt, HALF ? 7 : 12);
+        TS = CTS > 0 ? CTS : sp.ts;
+        RS = CTS > 0 ? slots / CTS : sp.rs;
         if (tid < 0 || tid / col >= TS * RS) {
             q = y = 0;
             t0 = g.Lt;
             r0 = g.nrep;
         } else {
-            q = tid % W();
-            y = (tid / W()) % Ly();
+            q = first() + tid % wp;
+            y = (tid / wp) % Ly();
             t0 = (tid / col) % TS;
             r0 = (tid / col) / TS;
         }
@@ -296,9 +321,11 @@ struct Traj {
         edge = edge_of(!rot ? t0 : t0 == 0 ? Lt() - 1 : t0 - 1);
         tb = rot ? t0 - 1 + step() : (step() == 1 ? 2 : t0 + 2);
         const int end = rot ? Lt() - 1 : Lt();
-        n_bulk = tb < end ? (end - tb - 1) / step() + 1 : 0;
-        up_last = 4 * rowW() *
-                  (!rot && tb + (n_bulk - 1) * step() == Lt() - 1 ? -(Lt() - 1) : 1);
+        const int n = tb < end ? (end - tb - 1) / step() + 1 : 0;
+        // every slot has n_all or (L_t and L even) n_all + 1 bulk rows
+        n_all = (rot ? (Lt() + step() - 1) / step() - 1 : n) - 1;
+        has_last = n > n_all;
+        up_last = 4 * rowW() * (!rot && tb + (n - 1) * step() == Lt() - 1 ? -(Lt() - 1) : 1);
     }
 
     // Flip bits of a word: s = nibble-wise sums of the neighbours of spin -1.
@@ -306,9 +333,9 @@ struct Traj {
                                               const uint4& ub) const
     {
         if constexpr (PAIR) {
-            return accept_pairs(s + own * 8u, ua, ub, tab);
+            return accept_pairs<HALF>(s + own * 8u, ua, ub, tab);
         } else {
-            return flips_of_counts<D>(s, own, count8<D>(ua, ub, J.tb));
+            return flips_of_counts<D>(s, own, count8<D, HALF>(ua, ub, J.tb));
         }
     }
 
@@ -369,6 +396,12 @@ struct Traj {
         const uint64_t q1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ x.c3k);
         return philox_from<2>((uint32_t)(q1 >> 32) ^ x.lo1k, (uint32_t)q1,
                               x.h0k ^ (uint32_t)p0, x.l0, K);
+    }
+
+    // The word's second block; a half word has none.
+    __device__ __forceinline__ uint4 second(uint64_t p0, const Stream& x) const
+    {
+        return HALF ? make_uint4(0u, 0u, 0u, 0u) : draw(p0 + kPhiloxM0, x);
     }
 
     // Site jl of a cut-row word that switches during the protocol: couplings
@@ -465,7 +498,8 @@ struct Traj {
 #pragma unroll 1
             for (int jl = k.jlo; jl < jhi; ++jl)
                 f = (f & ~(0xFu << (4 * jl))) |
-                    switched_site(jl, own, self_w, glue_w, s, word8(ua, ub, jl), P, dE);
+                    switched_site(jl, own, self_w, glue_w, s,
+                                  HALF ? word_of(ua, jl) : word8(ua, ub, jl), P, dE);
         }
         if (!FAST) f &= vmask;
         st(own_b, own_b + w4, own ^ f, 9);
@@ -477,13 +511,12 @@ struct Traj {
     __device__ __forceinline__ void bulk_rows(A own_b, A oth, int w4, uint64_t p0, int p, XShift x,
                                               const Stream& st) const
     {
-        int n = n_bulk;
         const uint64_t dp = (uint64_t)kPhiloxM0 * (uint32_t)(step() * Ly() * G());
         const int stride = step() * rowW() * 4;
         A own = own_b + w4, o = oth + w4;
         auto row = [&](int up) {
             const uint4 ua = draw(p0, st);
-            const uint4 ub = draw(p0 + kPhiloxM0, st);
+            const uint4 ub = second(p0, st);
             bulk_row(own_b, oth, own, o, up, x, ua, ub);
             p0 += dp;
             own += stride;
@@ -491,20 +524,44 @@ struct Traj {
             if (ODD) x = xshift(p ^= 1);
         };
         int up = 4 * rowW();
-        if constexpr (CLT > 0 && CTS > 2 && CLT % CTS == 0) {
-#pragma unroll
-            for (int k = 1; k < CLT / CTS; ++k) row(up);
-        } else {
-            // four rows per pass; the last row, whose t + 1 row may wrap
-            // around, is one of the single rows that follow
+        if constexpr (CLT > 0 && CTS > 2 && CLT % (2 * CTS) == 0) {
+            // two replicas a whole number of bank rows apart: the second one
+            // runs its bulk rows one step later around, so that the two
+            // fall on different banks
+            constexpr int N = CLT / CTS - 1;
+            static_assert(N % 2 == 1, "");
+            if (r0) {
+                p0 += dp;
+                own += stride;
+                o += stride;
+            }
 #pragma unroll 1
-            for (; n > 4; n -= 4) {
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int k = 0; k < N / 2; ++k) row(up);
+            }
+            if (r0) {
+                p0 -= N * dp;
+                own -= N * stride;
+                o -= N * stride;
+            }
+            row(up);
+        } else {
+            // n_all rows that every slot has, four per pass and then singly,
+            // so that a warp's slots do not diverge; then the last row, which
+            // some slots lack and whose t + 1 row may wrap around
+            int n = n_all;
+#pragma unroll 1
+            for (; n >= 4; n -= 4) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i) row(up);
             }
 #pragma unroll 1
-            for (; n > 0; --n) {
-                if (n == 1) up = up_last;
+            for (; n >= 0; --n) {
+                if (n == 0) {
+                    if (!has_last) break;
+                    up = up_last;
+                }
                 row(up);
             }
         }
@@ -535,7 +592,7 @@ struct Traj {
             auto first = [&](const Edge& e, const Cut& k, const XShift& x) {
                 const uint64_t p0 = (uint64_t)kPhiloxM0 * (cr + (uint32_t)(e.t * Ly() * G()));
                 const uint4 ua = draw(p0, st);
-                const uint4 ub = draw(p0 + kPhiloxM0, st);
+                const uint4 ub = second(p0, st);
                 edge_row(own_b, oth, 4 * (wr + e.t * rw), e, k, r, x, ua, ub, P, dE);
             };
             if (rot) {
@@ -632,29 +689,38 @@ struct Course {
         left = resume ? 0 : J.n_therm;
         P = StepState{-1, J.dir > 0 ? J.g0 : J.g1, 0, 0, J.tcut, false};
     }
-    // The next sweep's state for row y; false after the last one.
-    __device__ __forceinline__ bool next(int y)
+    // To the next sweep; false after the last one.
+    __device__ __forceinline__ bool next()
     {
         if (left == 0) {
             if (++k >= J.k_end) return false;
             left = J.n_sweep;
-            // protocol 2: only column y = k / den moves; the columns before it
-            // sit at the end geometry, the ones after it at the start geometry
-            const int ya = J.prot == 2 ? k / J.den : 0;
-            const int kp = k + 1 - ya * J.den;
+            const int kp = k + 1 - active() * J.den;
             P.w_self = J.dir > 0 ? J.den - kp : kp;
             P.w_glue = J.dir > 0 ? kp : J.den - kp;
             P.k = k;
             P.lg = J.g0;
             P.tk = J.tcut + (size_t)k * (8 * D);
             P.record = true;
-            if (J.prot == 2 && y != ya) {
-                P.k = -1;
-                P.lg = (y < ya) == (J.dir > 0) ? J.g1 : J.g0;
-            }
         }
         --left;
         return true;
+    }
+    // Protocol 2: only column y = active() moves at step k >= 0.
+    __device__ __forceinline__ int active() const { return J.prot == 2 ? k / J.den : 0; }
+    // The sweep's state for row y (protocol 2: the columns before the active one
+    // sit at the end geometry, the ones after it at the start geometry).
+    __device__ __forceinline__ StepState of_row(int y) const
+    {
+        StepState s = P;
+        if (D == 3 && J.prot == 2 && P.k >= 0) {
+            const int ya = active();
+            if (y != ya) {
+                s.k = -1;
+                s.lg = (y < ya) == (J.dir > 0) ? J.g1 : J.g0;
+            }
+        }
+        return s;
     }
 };
 
@@ -743,7 +809,7 @@ __device__ __forceinline__ int run_rows(const Tr& tr, const Geom& g, const Philo
         bar();
     };
 #pragma unroll 1
-    while (C.next(0)) {
+    while (C.next()) {
         if (C.P.lg != lg) {
             lg = C.P.lg;
             m[0] = cut ? tr.glue_mask(lg, tr.t0 & 1) : 0u;
@@ -764,31 +830,40 @@ __device__ __forceinline__ int run_rows(const Tr& tr, const Geom& g, const Philo
 // that makes W = (beta/N) W_int).
 // sin: the stored state to start from when J.k_begin > 0 or J.start_in (else unused).
 // ROW: the team has a thread per word (run_rows).
-template <int D, bool FAST, bool PAIR, bool HBM, int CW, int CLY, bool ROW = false, int CLT = 0,
+template <int D, int KIND, bool PAIR, bool HBM, int CW, int CLY, bool ROW = false, int CLT = 0,
           int CTS = 0, class Bar>
 __device__ __forceinline__ int run_trajectory(const Geom& g, const PhiloxKeys& K, const TeamJob& J,
                                               long long traj, uint32_t* S_team, const uint2* tab,
                                               int tid, int nthr, Bar bar,
                                               const int8_t* sin = nullptr)
 {
-    const Traj<D, FAST, PAIR, HBM, CW, CLY, CLT, CTS> tr(g, S_team, tab, J, K, (uint32_t)traj,
-                                                         tid, nthr);
+    constexpr bool TAIL = KIND == kHalfTail;
+    const Traj<D, KIND == kWhole, PAIR, HBM, CW, CLY, CLT, CTS, TAIL ? kWholeWords : kAllWords> tr(
+        g, S_team, tab, J, K, (uint32_t)traj, tid, nthr);
+    // rows that end in half a word: the half words have threads of their own
+    const Traj<D, false, PAIR, HBM, CW, CLY, CLT, CTS, kTailWords> tail(g, S_team, tab, J, K,
+                                                                       (uint32_t)traj, tid, nthr);
     if (J.k_begin > 0 || J.start_in) {
-        if (tid >= 0) tr.import_spins(sin);
+        if (tid >= 0) {
+            tr.import_spins(sin);
+            if (TAIL) tail.import_spins(sin);
+        }
     } else {
         tr.hot_start();
+        if (TAIL) tail.hot_start();
     }
     bar();
     if constexpr (ROW) {
-        return run_rows<FAST>(tr, g, K, J, bar);
+        return run_rows<KIND == kWhole>(tr, g, K, J, bar);
     } else {
         int dE = 0;
         Course<D> C(J);
 #pragma unroll 1
-        while (C.next(tr.y)) {
+        while (C.next()) {
 #pragma unroll 1
             for (int c = 0; c < 2; ++c) {
-                tr.half_sweep(c, C.s, C.P, dE);
+                tr.half_sweep(c, C.s, C.of_row(tr.y), dE);
+                if (TAIL) tail.half_sweep(c, C.s, C.of_row(tail.y), dE);
                 bar();
                 C.P.record = false;
             }

@@ -4,20 +4,24 @@
 namespace jz {
 
 // Shapes with compile-time row geometry: L = 16 and 64 (GW = 1, 4); the L =
-// L_t = 64 warp teams (eight time slices per thread) also fix L_t and the slice
-// step.  Every other shape runs the generic instantiation.
+// L_t = 64 warp teams of an even number of replicas (four slices by two replicas
+// at a time; 31 x 1024 trajectories 533 ms with eight slices of one, 527 so) also
+// fix L_t and the slice step.  Every other shape runs the generic instantiation.
 TrajFn select_traj2d(const Geom& g, const LaunchShape& sh, bool hbm, bool pair)
 {
-    const bool fast = (g.Lh % 8) == 0;
+    const int kind = row_kind(g, sh);
     if (!pair)
-        return fast ? pick_traj<2, true, false, 0, 0>(sh, hbm)
-                    : pick_traj<2, false, false, 0, 0>(sh, hbm);
-    if (fast && g.GW == 4 && g.Lt == 64 && sh.warp && sh.team_threads == 32 && !hbm)
-        return pick_traj<2, true, true, 4, 1, 64, 8>(sh, hbm);
-    if (fast && g.GW == 4) return pick_traj<2, true, true, 4, 1>(sh, hbm);
-    if (fast && g.GW == 1) return pick_traj<2, true, true, 1, 1>(sh, hbm);
-    return fast ? pick_traj<2, true, true, 0, 0>(sh, hbm)
-                : pick_traj<2, false, true, 0, 0>(sh, hbm);
+        return kind == kWhole    ? pick_traj<2, kWhole, false, 0, 0>(sh, hbm)
+               : kind == kRagged ? pick_traj<2, kRagged, false, 0, 0>(sh, hbm)
+                                 : pick_traj<2, kHalfTail, false, 0, 0>(sh, hbm);
+    if (kind == kWhole && g.GW == 4 && g.Lt == 64 && g.nrep % 2 == 0 && sh.warp &&
+        sh.team_threads == 32 && !hbm)
+        return pick_traj<2, kWhole, true, 4, 1, 64, 4>(sh, hbm);
+    if (kind == kWhole && g.GW == 4) return pick_traj<2, kWhole, true, 4, 1>(sh, hbm);
+    if (kind == kWhole && g.GW == 1) return pick_traj<2, kWhole, true, 1, 1>(sh, hbm);
+    return kind == kWhole    ? pick_traj<2, kWhole, true, 0, 0>(sh, hbm)
+           : kind == kRagged ? pick_traj<2, kRagged, true, 0, 0>(sh, hbm)
+                             : pick_traj<2, kHalfTail, true, 0, 0>(sh, hbm);
 }
 
 cudaError_t bounds_status_traj2d(unsigned int out[2], bool clear)

@@ -7,13 +7,15 @@ namespace jz {
 // runs the generic instantiation.
 TrajFn select_traj3d(const Geom& g, const LaunchShape& sh, bool hbm, bool pair)
 {
-    const bool fast = (g.Lh % 8) == 0;
+    const int kind = row_kind(g, sh);
     if (!pair)
-        return fast ? pick_traj<3, true, false, 0, 0>(sh, hbm)
-                    : pick_traj<3, false, false, 0, 0>(sh, hbm);
-    if (fast && g.GW == 1 && g.Ly == 16) return pick_traj<3, true, true, 1, 16>(sh, hbm);
-    return fast ? pick_traj<3, true, true, 0, 0>(sh, hbm)
-                : pick_traj<3, false, true, 0, 0>(sh, hbm);
+        return kind == kWhole   ? pick_traj<3, kWhole, false, 0, 0>(sh, hbm)
+               : kind == kRagged ? pick_traj<3, kRagged, false, 0, 0>(sh, hbm)
+                                 : pick_traj<3, kHalfTail, false, 0, 0>(sh, hbm);
+    if (kind == kWhole && g.GW == 1 && g.Ly == 16) return pick_traj<3, kWhole, true, 1, 16>(sh, hbm);
+    return kind == kWhole   ? pick_traj<3, kWhole, true, 0, 0>(sh, hbm)
+           : kind == kRagged ? pick_traj<3, kRagged, true, 0, 0>(sh, hbm)
+                             : pick_traj<3, kHalfTail, true, 0, 0>(sh, hbm);
 }
 
 cudaError_t bounds_status_traj3d(unsigned int out[2], bool clear)

@@ -32,7 +32,7 @@ constexpr int kMaxTeams = 64;
 // to 32 warps) the 2D L = 64 scan (31 x 1024 trajectories) took 555, 560, 587
 // and 593 ms against 558 ms uncapped, the 3D L = 24, L_t = 96 lattice 132, 141,
 // 154 and 154 ms against 133 ms.
-template <int D, bool FAST, bool PAIR, int CW, int CLY, bool WARP, bool HBM, int CLT = 0,
+template <int D, int KIND, bool PAIR, int CW, int CLY, bool WARP, bool HBM, int CLT = 0,
           int CTS = 0>
 __global__ void __launch_bounds__(512, 1)
 traj_kernel(const Geom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, int n_jobs,
@@ -64,15 +64,15 @@ traj_kernel(const Geom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
     int dE;
     // The one-row path is compiled into the 2D GW = 1 variant (L = 16), the
     // only lattice whose warp team can hold a thread per word.
-    constexpr bool kRow = D == 2 && FAST && CW == 1 && WARP;
+    constexpr bool kRow = D == 2 && KIND == kWhole && CW == 1 && WARP;
     if (kRow && sh.team_threads == g.NR * g.GW)
-        dE = run_trajectory<D, FAST, PAIR, HBM, CW, CLY, kRow>(g, K, tj, traj, St, s_tab, tid,
+        dE = run_trajectory<D, KIND, PAIR, HBM, CW, CLY, kRow>(g, K, tj, traj, St, s_tab, tid,
                                                                sh.team_threads, WarpBarrier{}, sin);
     else if (WARP)
-        dE = run_trajectory<D, FAST, PAIR, HBM, CW, CLY, false, CLT, CTS>(
+        dE = run_trajectory<D, KIND, PAIR, HBM, CW, CLY, false, CLT, CTS>(
             g, K, tj, traj, St, s_tab, tid, sh.team_threads, WarpBarrier{}, sin);
     else
-        dE = run_trajectory<D, FAST, PAIR, HBM, CW, CLY>(g, K, tj, traj, St, s_tab, tid,
+        dE = run_trajectory<D, KIND, PAIR, HBM, CW, CLY>(g, K, tj, traj, St, s_tab, tid,
                                                          sh.team_threads, CtaBarrier{}, sin);
     if (has && dE != 0) atomicAdd(&s_work[tm], dE);
     __syncthreads();
@@ -87,13 +87,13 @@ traj_kernel(const Geom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
 using TrajFn = void (*)(const Geom, const PhiloxKeys, const JobDesc*, int, const LaunchShape,
                        uint32_t*);
 
-template <int D, bool FAST, bool PAIR, int CW, int CLY, int CLT = 0, int CTS = 0>
+template <int D, int KIND, bool PAIR, int CW, int CLY, int CLT = 0, int CTS = 0>
 TrajFn pick_traj(const LaunchShape& sh, bool hbm)
 {
-    return hbm ? (sh.warp ? traj_kernel<D, FAST, PAIR, CW, CLY, true, true>
-                          : traj_kernel<D, FAST, PAIR, CW, CLY, false, true>)
-               : (sh.warp ? traj_kernel<D, FAST, PAIR, CW, CLY, true, false, CLT, CTS>
-                          : traj_kernel<D, FAST, PAIR, CW, CLY, false, false>);
+    return hbm ? (sh.warp ? traj_kernel<D, KIND, PAIR, CW, CLY, true, true>
+                          : traj_kernel<D, KIND, PAIR, CW, CLY, false, true>)
+               : (sh.warp ? traj_kernel<D, KIND, PAIR, CW, CLY, true, false, CLT, CTS>
+                          : traj_kernel<D, KIND, PAIR, CW, CLY, false, false>);
 }
 
 // The instantiation that runs lattices g in shape sh (pair: with the
