@@ -275,8 +275,8 @@ int jarzynski_run_batch(ising_ctx* ctx, const jz_params* jobs, int n_jobs,
  *   est_out       caller-owned DEVICE buffer of 3 n_jobs doubles (nullable):
  *                 per job ln <e^-W>, Delta S_2 and its jackknife error, as
  *                 estimator_reduce with 32 blocks
- *   cta_threads   CTA size of the persistent kernel (0 = autotune: each of
- *                 256, 288, 384, 512 is timed on a reduced copy of the batch)
+ *   cta_threads   CTA size of the persistent kernel (0 = the one of 256, 288,
+ *                 384 and 512 whose schedule of the batch is the shortest)
  * The plan keeps its own device tables (charged to the context's budget) and
  * records the pointers it was given: they must stay valid while it is used.
  * Each job's results are bit-identical to running it alone with

@@ -6,9 +6,11 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <mutex>
 #include <new>
+#include <queue>
 #include <tuple>
 #include <vector>
 
@@ -1300,29 +1302,37 @@ cudaError_t launch_persistent(const BatchJob* jobs, const int2* items, int n_ite
 cudaError_t launch_estimator_batch(const EstJob* jobs, int n_jobs, double* out, cudaStream_t st);
 }  // namespace jz
 
+// A half-sweep's time in a CTA team or warp team of shape sh (sweep_cost's unit).
+double team_time(const jz::Geom& g, const jz::LaunchShape& sh)
+{
+    jz::RowKind kind;
+    return jz::sweep_cost(g, sh.team_threads, &kind) + (sh.warp ? 0.0 : 2 * kBarrier);
+}
+
 // A job's layout inside the plan's CTAs of cta threads: the warp teams of
 // shape_for, or one team of the whole CTA when that takes less of the CTA's time
-// per trajectory (sweep_cost).  A large lattice leaves most warps of a warp-team
-// CTA idle -- 2D L = 128 fits seven 32 KB lattices in a 384-thread CTA -- and
-// its shared memory would then set every CTA's, one CTA per SM; as one team it
-// holds one lattice.
-jz::LaunchShape plan_shape(const jz::Geom& g, int cta)
+// per trajectory, or when the warp teams' lattices take more than the CTA's share
+// of shared memory with `resident` threads on the SM.  The largest layout sets
+// every CTA's shared memory: 2D L = 128 holds eight 16 KB lattices in a 256-thread
+// CTA as warp teams, and the plan would run one such CTA, eight warps, per SM.
+// resident = kOneTeam leaves no share: one team wherever a warp's worth of
+// threads can work, the layout of short items for plans of few trajectories.
+constexpr int kOneTeam = 1 << 24;
+jz::LaunchShape plan_shape(const jz::Geom& g, int cta, int resident)
 {
     const jz::LaunchShape w = shape_for(g, cta);
     const int col = g.GW * g.Ly;
     const int ts = std::min(cta / col, g.Lt);
     if (ts < 1 || col * ts < 32) return w;
-    auto busy = [&](const jz::LaunchShape& sh) {
-        jz::RowKind kind;
-        return sh.teams /
-               (jz::sweep_cost(g, sh.team_threads, &kind) + (sh.warp ? 0.0 : 2 * kBarrier));
-    };
     jz::LaunchShape c{};
     c.team_threads = col * ts;
     c.teams = 1;
     c.cta_threads = col * ts;
     c.warp = 0;
-    return busy(c) > kKeepMargin * busy(w) ? c : w;
+    const size_t lat = jz::traj_smem_bytes(g);
+    const size_t share = jz::kMaxSmemPerCta * (size_t)cta / std::max(cta, resident);
+    if (w.teams * lat + jz::kPairReserve > share && w.teams > 1) return c;
+    return w.teams / team_time(g, w) * kKeepMargin < 1.0 / team_time(g, c) ? c : w;
 }
 
 struct jz_plan {
@@ -1383,9 +1393,86 @@ void plan_release(jz_plan* pl)
     delete pl;
 }
 
+// Chooses a plan's CTA size (*cta = 0: open; 0 again if none can run the jobs) and the threads per SM that its layouts make room for: the
+// shortest schedule, each candidate's items handed out as the kernel does, longest
+// first to the CTA that is free first, in shape_score's units (3 warps per SM
+// sub-partition take 0.78 of the time of 4).  27 jobs, 2D L = 32 .. 128 and 3D L = 8
+// .. 24: 49.8 ms with the 384 threads it takes; 55.4 ms with the 256 that a trial
+// run of a sixteenth of the trajectories chose, which saw neither the waves nor
+// the tail of the full plan.  Its 2D L = 96 jobs alone: 13.6 -> 3.8 ms (one team
+// per CTA).
+int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
+{
+    int dev = 0, n_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return ISING_ERR_CUDA;
+    std::vector<int> sizes = {256, 288, 384, 512};
+    if (*cta > 0) sizes = {*cta};
+    double best = 1e300;
+    *cta = 0;
+    for (const int cand : sizes)
+        for (const int res : {512, 384, kOneTeam}) {
+            std::vector<std::pair<double, long long>> items;   // time, how many
+            size_t smem = 0;
+            bool ok = true, pair = true;
+            double sum = 0.0;
+            long long n = 0;
+            for (int j = 0; j < n_jobs && ok; ++j) {
+                const jz_params& p = jobs[j];
+                if (p.update == 1) continue;
+                const jz::Geom g = make_geom(p.d, p.L, p.L_t, nrep_of(p));
+                ok = threads_fit(g) && g.GW * g.Ly <= cand;
+                if (!ok) break;
+                const jz::LaunchShape sh = plan_shape(g, cand, res);
+                const size_t sm = sh.teams * jz::traj_smem_bytes(g);
+                ok = shape_fits(g) && sh.team_threads <= cand &&
+                     !(sh.warp && sh.cta_threads > cand) && sm <= jz::kMaxSmemPerCta;
+                smem = std::max(smem, sm);
+                pair = pair && jz::traj_pairs(g, sh.teams, false);
+                const double t =
+                    team_time(g, sh) * ((double)p.n_therm + (double)p.n_step * p.n_sweep);
+                const long long c = (p.n_traj + sh.teams - 1) / sh.teams;
+                items.push_back({t, c});
+                sum += t * c;
+                n += c;
+            }
+            if (!ok) continue;
+            if (pair) smem += jz::kPairTable * sizeof(uint2);
+            int per_sm = 0;
+            if (jz::persistent_prepare(pair, smem, cand, &per_sm) != cudaSuccess || per_sm < 1) {
+                cudaGetLastError();
+                continue;
+            }
+            const long long grid = std::min((long long)per_sm * n_sm, n);
+            double span = sum / grid;
+            if (n <= 20000) {   // beyond that the tail is short
+                std::sort(items.rbegin(), items.rend());
+                std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+                for (long long i = 0; i < grid; ++i) free_at.push(0.0);
+                span = 0.0;
+                for (const auto& it : items)
+                    for (long long i = 0; i < it.second; ++i) {
+                        const double end = free_at.top() + it.first;
+                        free_at.pop();
+                        free_at.push(end);
+                        span = std::max(span, end);
+                    }
+            }
+            const int wc = (cand + 31) / 32;
+            span *= ((grid + n_sm - 1) / n_sm * wc + 3) / 4 + 0.5;
+            if (span < best) {
+                best = span;
+                *cta = cand;
+                *resident = res;
+            }
+        }
+    return ISING_OK;
+}
+
 // Builds (not captures) a plan for a fixed CTA size.
 int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const* work_outs,
-               double* est_out, int cta, jz_plan** out)
+               double* est_out, int cta, int resident, jz_plan** out)
 {
     jz_plan* pl = new (std::nothrow) jz_plan();
     if (!pl) return ISING_ERR_NOMEM;
@@ -1454,7 +1541,7 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
         jz::BatchJob& B = bj[j];
         B.g = make_geom(p.d, p.L, p.L_t, nrep_of(p));
         B.D = p.d;
-        B.sh = plan_shape(B.g, cta);
+        B.sh = plan_shape(B.g, cta, resident);
         B.kind = jz::row_kind(B.g, B.sh);
         B.lattice_words = 2 * B.g.NR * B.g.GW;
         if (!shape_fits(B.g) || B.sh.team_threads > cta || (B.sh.warp && B.sh.cta_threads > cta)) {
@@ -1526,14 +1613,12 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
             therm_bytes += (size_t)p.n_traj * (size_t)(B.g.nrep * p.L_t * B.g.Ly * p.L);
             J.start_in = 1;
         }
-        const double per_traj = (double)(B.g.nrep * p.L_t * B.g.Ly * p.L) *
-                                ((double)p.n_therm + (double)p.n_step * p.n_sweep);
-        for (int lo = 0; lo < p.n_traj; lo += B.sh.teams) {
-            const int cnt = std::min(B.sh.teams, p.n_traj - lo);
-            items.push_back({per_traj * cnt, make_int2(j, lo)});
-        }
+        const double time = team_time(B.g, B.sh) *
+                            ((double)p.n_therm + (double)p.n_step * p.n_sweep);
+        for (int lo = 0; lo < p.n_traj; lo += B.sh.teams)
+            items.push_back({time, make_int2(j, lo)});
     }
-    // largest items first
+    // longest items first
     std::stable_sort(items.begin(), items.end(),
                      [](const std::pair<double, int2>& a, const std::pair<double, int2>& b) {
                          return a.first > b.first;
@@ -1721,48 +1806,17 @@ int jz_plan_create(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* c
     }
     if (est_out && !is_device_ptr(est_out)) return ISING_ERR_ARG;
     int rc;
-    int cta = cta_threads;
+    int cta = cta_threads, resident = 512;
     bool any_metropolis = false;
     for (int j = 0; j < n_jobs; ++j) any_metropolis |= jobs[j].update == 0;
-    if (cta == 0 && !any_metropolis) cta = 256;   // nothing runs in the persistent kernel
-    if (cta == 0) {
-        // autotune on a reduced copy: 1/16 of the trajectories, 8 + 8 sweeps
-        std::vector<jz_params> small(jobs, jobs + n_jobs);
-        for (auto& p : small) {
-            p.n_traj = std::max(1, p.n_traj / 16);
-            p.n_therm = 8;
-            p.n_step = 8;
-            p.n_sweep = 1;
-        }
-        cudaEvent_t e0, e1;
-        if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
-            return ISING_ERR_CUDA;
-        float best_ms = 1e30f;
-        for (int cand : {256, 288, 384, 512}) {
-            jz_plan* pl = nullptr;
-            if (plan_build(ctx, small.data(), n_jobs, work_outs, nullptr, cand, &pl)) continue;
-            float ms = 1e30f;
-            if (!plan_enqueue(pl)) {
-                cudaEventRecord(e0, ctx->stream);
-                if (!plan_enqueue(pl)) {
-                    cudaEventRecord(e1, ctx->stream);
-                    if (cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-                }
-            }
-            cudaStreamSynchronize(ctx->stream);
-            cudaGetLastError();
-            plan_release(pl);
-            if (ms < best_ms) {
-                best_ms = ms;
-                cta = cand;
-            }
-        }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
+    if (any_metropolis) {
+        if ((rc = plan_cta(jobs, n_jobs, &cta, &resident))) return rc;
         if (cta == 0) return ISING_ERR_UNSUPPORTED;
+    } else if (cta == 0) {
+        cta = 256;   // nothing runs in the persistent kernel
     }
     jz_plan* pl = nullptr;
-    if ((rc = plan_build(ctx, jobs, n_jobs, work_outs, est_out, cta, &pl))) return rc;
+    if ((rc = plan_build(ctx, jobs, n_jobs, work_outs, est_out, cta, resident, &pl))) return rc;
     if ((rc = plan_capture(pl))) {
         plan_release(pl);
         return rc;

@@ -72,3 +72,25 @@ def test_half_words_in_a_persistent_plan(lib):
             np.testing.assert_array_equal(ws[i].cpu().numpy(), Wo)
     finally:
         jz.ising_replica_free(c)
+
+
+# warp teams whose lattices take more than the CTA's share of shared memory, and
+# few trajectories: one team per CTA; many: warp teams
+@pytest.mark.parametrize("cta", [0, 256, 512])
+@pytest.mark.parametrize("n_traj", [3, 80])
+def test_plan_layouts(lib, cta, n_traj):
+    c = jz.ising_replica_init(0, 0, None)
+    shapes = [(2, 128, 128), (2, 96, 96), (2, 32, 32), (3, 12, 12)]
+    jobs = [jz.make_params(d, L, L_t, 0.3, 3, 2, 1, n_traj, 99, n_therm=1)
+            for d, L, L_t in shapes]
+    ws = [torch.empty(n_traj, dtype=torch.int64, device="cuda") for _ in jobs]
+    try:
+        plan = jz.jz_plan_create(c, jobs, ws, None, cta)
+        jz.jz_plan_launch(plan)
+        jz.ising_sync(c)
+        jz.jz_plan_free(plan)
+        for w, (d, L, L_t) in zip(ws, shapes):
+            Wo, _ = oracle.run(d, L, L_t, 0.3, 3, 2, 1, n_traj, 99, n_therm=1)
+            np.testing.assert_array_equal(w.cpu().numpy(), Wo)
+    finally:
+        jz.ising_replica_free(c)
