@@ -248,7 +248,7 @@ struct Traj {
     int r0, RS;               // first replica and replica step
     int d_qm, d_qp;           // byte offset of the x-shift neighbour word (p = 0 / 1)
     int d_ym, d_yp;           // byte offsets of the rows y-1 / y+1 (3D)
-    Edge edge;                // TS >= 3: the first row of each replica
+    Edge edge;                // TS >= 2: the first row of each replica
     int tb, n_all, up_last;   // first bulk row, the rows all slots have, the last one's t + 1 row
     bool has_last;            // one row more
     uint32_t vmask;           // nibbles of word q that hold sites (ragged rows)
@@ -571,8 +571,11 @@ struct Traj {
     // row t0 - 1 (slot 0 with L_t - 1): the two rows next to the cut and the row
     // whose t + 1 neighbour wraps around are all first rows, one instruction
     // stream for the whole team, and every other row is t0 - 1 + k TS with plain
-    // time neighbours.  With TS <= 2 the cut rows t = 0, 1 come first and the
-    // last bulk row wraps.
+    // time neighbours.  With TS <= 2 the cut rows t = 0, 1 come first, one per
+    // slot or both, and the last bulk row wraps.  TS = 2 takes its one row's
+    // geometry from `edge` in the kernels of whole words (3D L = 16: 159.4 -> 154.9
+    // ms); with ragged rows the registers cost more than they save (3D L = 22,
+    // 24: 1 % slower), and they recompute it.
     __device__ __forceinline__ void half_sweep(int c, uint32_t sweep, const StepState& P,
                                                int& dE) const
     {
@@ -582,7 +585,7 @@ struct Traj {
         const int ts = step();
         if (t0 >= lt) return;   // a thread without sites
         const Stream st = stream(c, sweep);
-        const bool rot = ts >= 3;
+        const bool one = ts >= (FAST ? 2 : 3);   // one edge row per replica, `edge`
         const Cut k0 = cut_of(edge, c, P);
         const XShift x0 = xshift(k0.p);
 #pragma unroll 1
@@ -595,7 +598,7 @@ struct Traj {
                 const uint4 ub = second(p0, st);
                 edge_row(own_b, oth, 4 * (wr + e.t * rw), e, k, r, x, ua, ub, P, dE);
             };
-            if (rot) {
+            if (one) {
                 first(edge, k0, x0);
             } else {
 #pragma unroll 1
@@ -609,7 +612,7 @@ struct Traj {
             const int w4 = 4 * (wr + tb * rw);
             const int p = (c + y + tb) & 1;
             if (CTS == 0 && (ts & 1)) bulk_rows<true>(own_b, oth, w4, p0, p, xshift(p), st);
-            else bulk_rows<false>(own_b, oth, w4, p0, p, rot ? x0 : xshift(p), st);
+            else bulk_rows<false>(own_b, oth, w4, p0, p, one ? x0 : xshift(p), st);
         }
     }
 

@@ -25,6 +25,8 @@ CASES = [
     (3, 18, 14, 7, 36 * 7, {}), (3, 18, 40, 9, 36 * 13, dict(n_replica=3)),
     (3, 20, 10, 11, 40 * 6, dict(protocol=2, direction=-1)), (3, 24, 18, 23, 48 * 5, {}),
     (3, 22, 12, 2, 44 * 11, dict(whole=True)),
+    (3, 16, 2, 5, 32, {}), (3, 16, 4, 8, 32, dict(n_replica=3)), (3, 16, 14, 9, 32, {}),
+    (3, 32, 4, 20, 64 * 2, {}), (3, 32, 10, 31, 64 * 2, dict(direction=-1)),
 ]
 
 
