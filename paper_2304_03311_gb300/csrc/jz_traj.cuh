@@ -40,8 +40,8 @@
 // at once, sums instead of XORs, one funnel shift per word, wrap-free bulk rows.
 // 2D L = 64: 134 instructions and 230 cycles per word (158 and 311 with one
 // lookup per site, four copies of the half-sweep whose code overflowed the
-// instruction cache, and a cut pass that recomputed its geometry):
-// 1.07e12 -> 1.53e12 spin updates/s on a scan of 31 x 1024 trajectories.
+// instruction cache, and a cut pass that recomputed its geometry): a scan of 31 x
+// 1024 trajectories 761 -> 527 ms, 1.02e12 -> 1.48e12 spin updates/s.
 //
 // The work increment is gathered inside the first colour-0 half-sweep of each
 // step: for every (r, y) exactly one of the switched sites (l, y, 0)^r and
@@ -56,7 +56,6 @@
 #include "jz_device.cuh"
 
 namespace jz {
-
 
 // ------------------------------------------------------------- acceptance --
 // A site with a anti-aligned neighbours (energy cost m = 2D - 2a) flips when

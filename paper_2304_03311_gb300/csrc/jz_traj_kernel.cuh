@@ -29,9 +29,9 @@ constexpr int kMaxTeams = 64;
 //
 // Registers: up to 128, i.e. 16 warps per SM.  The update is bound by the
 // arithmetic pipes, not by latency: capped at 96, 80, 72 and 64 registers (20
-// to 32 warps) the 2D L = 64 scan (31 x 1024 trajectories) took 555, 560, 587
-// and 593 ms against 558 ms uncapped, the 3D L = 24, L_t = 96 lattice 132, 141,
-// 154 and 154 ms against 133 ms.
+// to 32 warps) the 2D L = 64 scan (31 x 1024 trajectories) took 0.99, 1.00, 1.05
+// and 1.06 of the time uncapped, the 3D L = 24, L_t = 96 lattice 0.99, 1.06, 1.16
+// and 1.16.
 template <int D, int KIND, bool PAIR, int CW, int CLY, bool WARP, bool HBM, int CLT = 0,
           int CTS = 0>
 __global__ void __launch_bounds__(512, 1)
