@@ -52,6 +52,7 @@
 
 #include "jz_device.cuh"
 #include "jz_host.h"
+#include "jz_sw_words.cuh"
 
 namespace jz {
 
@@ -60,26 +61,6 @@ namespace {
 // Threads per CTA (one trajectory): 256 in 2D, 512 in 3D, whose extra +y
 // bonds make the union phase longer (measured on 2D 64^2 and 3D 16^3).
 __host__ __device__ constexpr int sw_threads(int D) { return D == 3 ? 512 : 256; }
-
-// Division by a fixed divisor d >= 1 for numerators n < 2^31 (Granlund and
-// Montgomery, PLDI'94): with s = ceil(log2 d) and m = floor(2^32 (2^s - d) / d)
-// + 1, n / d = (umulhi(m, n) + n) >> s.
-struct FastDiv {
-    uint32_t d, m, s;
-};
-
-FastDiv make_fastdiv(uint32_t d)
-{
-    uint32_t s = 0;
-    while ((1ull << s) < d) ++s;
-    const uint64_t m = (((1ull << s) - d) << 32) / d + 1;
-    return FastDiv{d, (uint32_t)m, s};
-}
-
-__device__ __forceinline__ uint32_t fdiv(uint32_t n, const FastDiv& f)
-{
-    return (__umulhi(f.m, n) + n) >> f.s;
-}
 
 struct SwGeom {
     int L, Lt, Ly;
@@ -125,6 +106,14 @@ __device__ __forceinline__ int spin_bit(const uint32_t* sp, int i, int V)
     return in_bounds(i, V, 20) ? (int)((sp[i >> 5] >> (i & 31)) & 1u) : 0;
 }
 
+// The spin bits as bits_at reads them.
+struct SpinBits {
+    const uint32_t* sp;
+    int V;
+    __device__ __forceinline__ bool has(int i) const { return in_bounds(i, V, 25); }
+    __device__ __forceinline__ uint32_t operator[](int w) const { return sp[w]; }
+};
+
 // Root of a with path halving: every visited node is re-pointed to its
 // grandparent.  A plain store is enough: the new parent is an ancestor of the
 // node, and a hook that a concurrent union made on that node is only ever
@@ -160,59 +149,11 @@ __device__ __forceinline__ void merge(int* lab, int a, int b, int V)
             a = b;
             b = t;
         }
+        if (!in_bounds(a, V, 21) || !in_bounds(b, V, 22)) return;
         const int old = atomicMin(&lab[a], b);
         if (old == a) return;
         a = old;
     }
-}
-
-// The word of bits o .. o + 31 of a bit array with a readable word on each side.
-__device__ __forceinline__ uint32_t bits_at(const uint32_t* a, int o)
-{
-    const int w = o >> 5;
-    return __funnelshift_r(a[w], a[w + 1], (uint32_t)o & 31u);
-}
-
-__device__ __forceinline__ int mod(int a, const FastDiv& f)
-{
-    return a - (int)(fdiv((uint32_t)a, f) * f.d);
-}
-
-// Bits lo .. hi - 1 of a word, clipped to it.
-__device__ __forceinline__ uint32_t bit_range(int lo, int hi)
-{
-    lo = max(lo, 0);
-    hi = min(hi, 32);
-    if (lo >= hi) return 0u;
-    return (hi == 32 ? 0xFFFFFFFFu : (1u << hi) - 1u) & ~((1u << lo) - 1u);
-}
-
-// The bits of a word whose sites' residues (the first one's: r) lie in [lo, hi)
-// of a period.
-__device__ __forceinline__ uint32_t residue_bits(int r, int period, int lo, int hi)
-{
-    uint32_t m = 0;
-    for (int b = -r; b < 32; b += period) m |= bit_range(b + lo, b + hi);
-    return m;
-}
-
-// What the thread-per-word phases need of word q: residues of its first site
-// (in its row, replica, slice) and the bits of its sites at their row's end.
-struct WordPos {
-    int base, x, v, u;
-    uint32_t valid, E;
-};
-template <int D>
-__device__ __forceinline__ WordPos word_pos(const SwGeom& g, int q)
-{
-    WordPos p;
-    p.base = 32 * q;
-    p.x = mod(p.base, g.dL);
-    p.v = mod(p.base, g.dVR);
-    p.u = D == 3 ? mod(p.base, g.dSL) : p.x;
-    p.valid = bit_range(0, g.V - p.base);
-    p.E = residue_bits(p.x, g.L, g.L - 1, g.L);
-    return p;
 }
 
 // Words a warp draws for at once in the grouped bond phase: at most 32, the same
@@ -286,7 +227,7 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
             bit = (int)(word_of(u, h & 3) >> 31);
         }
         const uint32_t m = __ballot_sync(0xFFFFFFFFu, bit);
-        if (lane == 0) sp[base >> 5] = m;
+        if (lane == 0 && in_bounds(base >> 5, g.VW, 26)) sp[base >> 5] = m;
     }
     __syncthreads();
 
@@ -389,23 +330,14 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
                 if (lane < count) {
                     const int q = first + lane;
                     const WordPos p = word_pos<D>(g, q);
-                    const uint32_t W = sp[q];
-                    // bits of the sites equal to their neighbour at +o (wrapping: o - wrap)
-                    auto equal = [&](uint32_t wraps, int o, int wrap) {
-                        uint32_t nb = 0;
-                        if (~wraps & p.valid) nb = bits_at(sp, p.base + o) & ~wraps;
-                        if (wraps) nb |= bits_at(sp, p.base + o - wrap) & wraps;
-                        return ~(W ^ nb) & p.valid;
-                    };
-                    const uint32_t X = rx & equal(p.E & p.valid, 1, g.L);
-                    m = X & ~p.E & 0x7FFFFFFFu;
+                    const uint32_t W = in_bounds(q, g.VW, 26) ? sp[q] : 0u;
+                    const SpinBits bits{sp, g.V};
+                    const uint32_t X = rx & equal_bits(bits, W, p.base, p.valid, p.x_end, 1, g.L);
+                    m = X & ~p.x_end & 0x7FFFFFFFu;
                     bx[q] = X & ~m;
-                    const uint32_t A = residue_bits(p.v, g.VR, g.VR - g.SL, g.VR) & p.valid;
-                    bt[q] = rt & equal(A, g.SL, g.VR);
-                    if (D == 3) {
-                        const uint32_t B = residue_bits(p.u, g.SL, g.SL - g.L, g.SL) & p.valid;
-                        by[q] = ry & equal(B, g.L, g.SL);
-                    }
+                    bt[q] = rt & equal_bits(bits, W, p.base, p.valid, p.t_end, g.SL, g.VR);
+                    if (D == 3)
+                        by[q] = ry & equal_bits(bits, W, p.base, p.valid, p.y_end, g.L, g.SL);
                     uint32_t G = 0;
                     rg &= p.valid;
                     while (rg) {
@@ -421,8 +353,8 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
                 // every site's label is its run's first site
                 for (int k = 0; k < count; ++k) {
                     const uint32_t brk = ~__shfl_sync(0xFFFFFFFFu, m, k) & ((1u << lane) - 1u);
-                    const int base = 32 * (first + k);
-                    if (base + lane < g.V) lab[base + lane] = base + 32 - __clz((int)brk);
+                    const int base = 32 * (first + k), i = base + lane;
+                    if (i < g.V && in_bounds(i, g.V, 27)) lab[i] = base + 32 - __clz((int)brk);
                 }
             }
         } else {
@@ -471,7 +403,7 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
             const uint32_t m = __ballot_sync(0xFFFFFFFFu, inw);
             const uint32_t brk = ~m & ((1u << lane) - 1u);
             const int start = brk ? 32 - __clz(brk) : 0;
-            if (i < g.V) lab[i] = base + start;
+            if (i < g.V && in_bounds(i, g.V, 27)) lab[i] = base + start;
             const uint32_t wx = __ballot_sync(0xFFFFFFFFu, ax && !inw);
             const uint32_t wt = __ballot_sync(0xFFFFFFFFu, at);
             const uint32_t wg = __ballot_sync(0xFFFFFFFFu, ag);
@@ -555,14 +487,14 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
                         if (up == root) break;
                         root = up;
                     }
-                    vl[i] = root;
+                    if (in_bounds(i, g.V, 27)) vl[i] = root;
                 } else {
                     root = find_root(vl, i, g.V);
                 }
-                f = (int)((fz[root >> 5] >> (root & 31)) & 1u);
+                f = in_bounds(root, g.V, 28) ? (int)((fz[root >> 5] >> (root & 31)) & 1u) : 0;
             }
             const uint32_t m = __ballot_sync(0xFFFFFFFFu, f);
-            if (lane == 0) sp[base >> 5] ^= m;
+            if (lane == 0 && in_bounds(base >> 5, g.VW, 26)) sp[base >> 5] ^= m;
         }
         __syncthreads();
     }
