@@ -306,11 +306,13 @@ jz::LaunchShape shape_for(const jz::Geom& g, int cta_threads)
 // three at a time run 4 % behind the model.  Up to kFewWaves waves the last wave,
 // CTAs that run with fewer others, counts by itself; in longer launches the CTAs
 // have drifted apart.  The busiest SM's CTAs decide: 256 trajectories on 152 SMs
-// last as long as two per SM.  Against the score before (active warps up to 16 per
-// SM x lanes owning a word x a barrier term), and with rows shared out by
-// split_rows: 2D L = 34 .. 240 and 3D L = 8 .. 36 run in 0.91 of the time on
-// average at 256 and 4096 trajectories (0.71 .. 1.03).  Negative when sh cannot
-// launch.
+// last as long as two per SM.  Only the launch's own trajectories count, not the
+// idle teams of a CTA that has more: one trajectory of 2D L = 160 takes 1.3 ms for
+// 200 sweeps as a team of 510 threads, 6.3 ms as one of four warp teams.  Against
+// the score before (active warps up to 16 per SM x lanes owning a word x a barrier
+// term), and with rows shared out by split_rows: 2D L = 34 .. 240 and 3D L = 8 .. 36
+// run in 0.91 of the time on average at 256 and 4096 trajectories (0.71 .. 1.03).
+// Negative when sh cannot launch.
 constexpr double kAlone = 1.0;     // a sub-partition's fixed part, in warps
 constexpr double kBarrier = 4.0;   // a CTA barrier's cost beside other CTAs (sweep_cost's unit)
 constexpr int kFewWaves = 6;
@@ -328,16 +330,16 @@ double shape_score(int d, const jz::Geom& g, const jz::LaunchShape& sh, long lon
     const int wc = (sh.cta_threads + 31) / 32;
     jz::RowKind kind;
     const double cost = jz::sweep_cost(g, sh.team_threads, &kind);
-    const double words = (double)g.NR * g.GW * sh.teams;
+    const double words = (double)g.NR * g.GW;   // of a trajectory
     auto time = [&](long long k) {   // of k resident CTAs
         return (cost + (sh.warp ? 0.0 : kBarrier * (1.0 + 1.0 / k))) *
                ((k * wc + 3) / 4 + kAlone + (wc == 5 && k > 1 ? 0.2 : 0.0));
     };
     const long long n_cta = (n_traj + sh.teams - 1) / sh.teams;
     const long long m = (n_cta + n_sm - 1) / n_sm;   // CTAs of the busiest SM
-    if (n_traj <= 0 || m >= kFewWaves * ctas) return ctas * words / time(ctas);
+    if (n_traj <= 0 || m >= kFewWaves * ctas) return ctas * sh.teams * words / time(ctas);
     const double t = (m / ctas) * time(ctas) + (m % ctas ? time(m % ctas) : 0.0);
-    return words * n_cta / n_sm / t;
+    return words * n_traj / n_sm / t;
 }
 
 // The shape a lattice in shared memory runs with when no CTA size is fixed.
