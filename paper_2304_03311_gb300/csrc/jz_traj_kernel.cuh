@@ -65,7 +65,7 @@ traj_kernel(const Geom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
     // The one-row path is compiled into the 2D GW = 1 variant (L = 16), the
     // only lattice whose warp team can hold a thread per word.
     constexpr bool kRow = D == 2 && KIND == kWhole && CW == 1 && WARP;
-    if (kRow && sh.team_threads == g.NR * g.GW)
+    if (kRow && one_row_team(g, sh))
         dE = run_trajectory<D, KIND, PAIR, HBM, CW, CLY, kRow>(g, K, tj, traj, St, s_tab, tid,
                                                                sh.team_threads, WarpBarrier{}, sin);
     else if (WARP)
