@@ -571,10 +571,10 @@ struct Traj {
     // whose t + 1 neighbour wraps around are all first rows, one instruction
     // stream for the whole team, and every other row is t0 - 1 + k TS with plain
     // time neighbours.  With TS <= 2 the cut rows t = 0, 1 come first, one per
-    // slot or both, and the last bulk row wraps.  TS = 2 takes its one row's
-    // geometry from `edge` in the kernels of whole words (3D L = 16: 159.4 -> 154.9
-    // ms); with ragged rows the registers cost more than they save (3D L = 22,
-    // 24: 1 % slower), and they recompute it.
+    // slot or both, and the last bulk row wraps.  From TS = 2 on a thread has one
+    // edge row per replica, whose geometry is `edge` (3D L = 16: 159.4 -> 154.9 ms;
+    // short lattices, L_t = 2, L = 4 .. 40: 0.79 .. 0.88 of the time); TS = 1
+    // recomputes that of its two rows.
     __device__ __forceinline__ void half_sweep(int c, uint32_t sweep, const StepState& P,
                                                int& dE) const
     {
@@ -584,7 +584,7 @@ struct Traj {
         const int ts = step();
         if (t0 >= lt) return;   // a thread without sites
         const Stream st = stream(c, sweep);
-        const bool one = ts >= (FAST ? 2 : 3);   // one edge row per replica, `edge`
+        const bool one = ts >= 2;   // one edge row per replica, `edge`
         const Cut k0 = cut_of(edge, c, P);
         const XShift x0 = xshift(k0.p);
 #pragma unroll 1
