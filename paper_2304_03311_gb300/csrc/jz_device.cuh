@@ -109,7 +109,12 @@ __host__ __device__ inline RowSplit split_rows(int slots, int nrep, int Lt, int 
 enum RowKind { kRagged = 0, kWhole = 1, kHalfTail = 2 };
 
 // A half-sweep's length with a team of nthr threads (split_rows' unit), and the
-// kind it takes: half words apart where that is shorter.
+// kind it takes: half words apart where that is shorter by more than the second pass
+// over the half-sweep costs, which takes about an edge row's extra to set up (few rows
+// per thread, 3D L = 18 .. 24, L_t = 2 .. 6, up to 152 trajectories: 0.82 .. 0.91 of the
+// time as one pass, though counted 5 shorter as two; 300 trajectories of 3D L = 18, L_t
+// = 4, where throughput counts, take 1.04).
+constexpr int kSecondPass = 8;
 __host__ __device__ inline int sweep_cost(const Geom& g, int nthr, RowKind* kind)
 {
     const int all = split_rows(nthr / (g.GW * g.Ly), g.nrep, g.Lt, 12).cost;
@@ -118,7 +123,7 @@ __host__ __device__ inline int sweep_cost(const Geom& g, int nthr, RowKind* kind
     const int whole =
         g.GW == 1 ? 0 : split_rows(nthr / ((g.GW - 1) * g.Ly), g.nrep, g.Lt, 12).cost;
     const int apart = whole + split_rows(nthr / g.Ly, g.nrep, g.Lt, 7).cost;
-    if (apart >= all) return all;
+    if (apart + (whole ? kSecondPass : 0) >= all) return all;
     *kind = kHalfTail;
     return apart;
 }
