@@ -109,12 +109,13 @@ __host__ __device__ inline RowSplit split_rows(int slots, int nrep, int Lt, int 
 enum RowKind { kRagged = 0, kWhole = 1, kHalfTail = 2 };
 
 // A half-sweep's length with a team of nthr threads (split_rows' unit), and the
-// kind it takes: half words apart where that is shorter by more than the second pass
-// over the half-sweep costs, which takes about an edge row's extra to set up (few rows
-// per thread, 3D L = 18 .. 24, L_t = 2 .. 6, up to 152 trajectories: 0.82 .. 0.91 of the
-// time as one pass, though counted 5 shorter as two; 300 trajectories of 3D L = 18, L_t
-// = 4, where throughput counts, take 1.04).
-constexpr int kSecondPass = 8;
+// kind it takes: half words apart where that is shorter.  In short half-sweeps, up to
+// six rows per thread (kShortSweep), a second pass over the half-sweep counts as well
+// (kSecondPass, an edge row's extra): up to 152 trajectories of 3D L = 18 .. 24, L_t = 2
+// .. 24, at 35 against 40 or 73 against 80 units, take 0.78 .. 0.95 of the time in one pass
+// (L = 22, 24, L_t = 6: 1.02); 300 of L = 18, L_t = 4, where throughput counts, 1.04.  3D L =
+// 36, 40, L_t = 16, at 109 against 112 units, take 1.05 in one pass.
+constexpr int kSecondPass = 8, kShortSweep = 80;
 __host__ __device__ inline int sweep_cost(const Geom& g, int nthr, RowKind* kind)
 {
     const int all = split_rows(nthr / (g.GW * g.Ly), g.nrep, g.Lt, 12).cost;
@@ -123,9 +124,8 @@ __host__ __device__ inline int sweep_cost(const Geom& g, int nthr, RowKind* kind
     const int whole =
         g.GW == 1 ? 0 : split_rows(nthr / ((g.GW - 1) * g.Ly), g.nrep, g.Lt, 12).cost;
     const int apart = whole + split_rows(nthr / g.Ly, g.nrep, g.Lt, 7).cost;
-    if (apart + (whole ? kSecondPass : 0) >= all) return all;
-    *kind = kHalfTail;
-    return apart;
+    if (apart + (whole && all <= kShortSweep ? kSecondPass : 0) < all) *kind = kHalfTail;
+    return all < apart ? all : apart;
 }
 __host__ __device__ inline RowKind row_kind(const Geom& g, const LaunchShape& sh)
 {

@@ -18,6 +18,7 @@ CASES = [
     (3, 24, 96, 192, HALF_TAIL), (3, 24, 24, 192, HALF_TAIL), (3, 20, 20, 120, HALF_TAIL),
     (3, 18, 2, 36, HALF_TAIL),                              # two rows per thread in one pass
     (2, 8, 8, 16, HALF_TAIL), (2, 2, 2, 4, HALF_TAIL),
+    (3, 36, 16, 432, HALF_TAIL), (3, 40, 20, 480, HALF_TAIL),   # throughput counts
     (3, 8, 8, 32, HALF_TAIL),                               # half words only: one pass
     (2, 64, 64, 32, WHOLE), (3, 28, 28, 112, RAGGED),       # none, and five to seven sites
 ]
