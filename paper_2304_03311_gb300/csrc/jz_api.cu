@@ -308,12 +308,16 @@ jz::LaunchShape shape_for(const jz::Geom& g, int cta_threads)
 // have drifted apart.  The busiest SM's CTAs decide: 256 trajectories on 152 SMs
 // last as long as two per SM.  Only the launch's own trajectories count, not the
 // idle teams of a CTA that has more: one trajectory of 2D L = 160 takes 1.3 ms for
-// 200 sweeps as a team of 510 threads, 6.3 ms as one of four warp teams.  Against
+// 200 sweeps as a team of 510 threads, 6.3 ms as one of four warp teams.  With at
+// most one CTA on any SM more warps hide more latency, and ties go to them (kOneCta):
+// three warps per sub-partition take 1.6 of what one takes, not twice as long (3D L =
+// 28, L_t = 6, up to 152 trajectories: 112 threads 0.43 ms, 336 threads 0.34).  Against
 // the score before (active warps up to 16 per SM x lanes owning a word x a barrier
 // term), and with rows shared out by split_rows: 2D L = 34 .. 240 and 3D L = 8 .. 36
 // run in 0.91 of the time on average at 256 and 4096 trajectories (0.71 .. 1.03).
 // Negative when sh cannot launch.
 constexpr double kAlone = 1.0;     // a sub-partition's fixed part, in warps
+constexpr double kOneCta = 0.05;    // more of it with one CTA per SM
 constexpr double kBarrier = 4.0;   // a CTA barrier's cost beside other CTAs (sweep_cost's unit)
 constexpr int kFewWaves = 6;
 double shape_score(int d, const jz::Geom& g, const jz::LaunchShape& sh, long long n_traj,
@@ -331,12 +335,13 @@ double shape_score(int d, const jz::Geom& g, const jz::LaunchShape& sh, long lon
     jz::RowKind kind;
     const double cost = jz::sweep_cost(g, sh.team_threads, &kind);
     const double words = (double)g.NR * g.GW;   // of a trajectory
-    auto time = [&](long long k) {   // of k resident CTAs
-        return (cost + (sh.warp ? 0.0 : kBarrier * (1.0 + 1.0 / k))) *
-               ((k * wc + 3) / 4 + kAlone + (wc == 5 && k > 1 ? 0.2 : 0.0));
-    };
     const long long n_cta = (n_traj + sh.teams - 1) / sh.teams;
     const long long m = (n_cta + n_sm - 1) / n_sm;   // CTAs of the busiest SM
+    auto time = [&](long long k) {   // of k resident CTAs
+        return (cost + (sh.warp ? 0.0 : kBarrier * (1.0 + 1.0 / k))) *
+               ((k * wc + 3) / 4 + kAlone + (m == 1 ? kOneCta : 0.0) +
+                (wc == 5 && k > 1 ? 0.2 : 0.0));
+    };
     if (n_traj <= 0 || m >= kFewWaves * ctas) return ctas * sh.teams * words / time(ctas);
     const double t = (m / ctas) * time(ctas) + (m % ctas ? time(m % ctas) : 0.0);
     return words * n_traj / n_sm / t;

@@ -26,3 +26,12 @@ def _shape(d, L, L_t, n_replica, n_traj):
 def test_a_lone_trajectory_gets_a_wide_team(L, L_t, n):
     sh = _shape(2, L, L_t, n, 1)
     assert sh["teams"] == 1 and sh["team_threads"] >= 256, sh
+
+
+# one CTA per SM: a slice per slot, six or more warps, beats a third of them with
+# three times the rows each
+@pytest.mark.parametrize("L", [28, 32])
+@pytest.mark.parametrize("n_traj", [1, 152])
+def test_few_trajectories_get_a_team_of_every_slice(L, n_traj):
+    sh = _shape(3, L, 6, 2, n_traj)
+    assert sh["team_threads"] == -(-L // 16) * L * 6, sh
