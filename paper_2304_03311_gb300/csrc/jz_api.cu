@@ -23,6 +23,19 @@ static_assert(sizeof(jz_params) == 80, "jz_params layout is part of the ABI");
 
 namespace jzh {
 
+// The estimate's three words, and beside them the scratch of the estimator's grid.
+constexpr size_t kEstBytes = 4 * sizeof(double);
+constexpr size_t kEstGridBytes = 64 + jz::kEstScratch;
+
+static void give_back(ising_ctx* ctx, DevBuf& b)
+{
+    cudaStreamSynchronize(ctx->stream);
+    cudaFree(b.ptr);
+    ctx->used -= b.bytes;
+    b.ptr = nullptr;
+    b.bytes = 0;
+}
+
 int ensure(ising_ctx* ctx, DevBuf& b, size_t bytes)
 {
     if (bytes <= b.bytes) return ISING_OK;
@@ -31,15 +44,15 @@ int ensure(ising_ctx* ctx, DevBuf& b, size_t bytes)
     if (ctx->budget && ctx->used + delta > ctx->budget) {
         want = bytes;
         delta = want - b.bytes;
+        // the estimator's scratch only makes it faster: others come first
+        if (ctx->used + delta > ctx->budget && &b != &ctx->est_out &&
+            ctx->est_out.bytes >= kEstGridBytes) {
+            give_back(ctx, ctx->est_out);
+            if (const int rc = ensure(ctx, ctx->est_out, kEstBytes)) return rc;
+        }
         if (ctx->used + delta > ctx->budget) return ISING_ERR_NOMEM;
     }
-    if (b.ptr) {
-        cudaStreamSynchronize(ctx->stream);
-        cudaFree(b.ptr);
-        ctx->used -= b.bytes;
-        b.ptr = nullptr;
-        b.bytes = 0;
-    }
+    if (b.ptr) give_back(ctx, b);
     if (cudaMalloc(&b.ptr, want) != cudaSuccess) {
         cudaGetLastError();
         return ISING_ERR_NOMEM;
@@ -801,7 +814,6 @@ void ising_replica_free(ising_ctx* ctx)
     for (DevBuf* b : {&ctx->tcut, &ctx->jobs, &ctx->work, &ctx->spins, &ctx->est_in,
                       &ctx->est_out, &ctx->lattice, &ctx->therm})
         if (b->ptr) cudaFree(b->ptr);
-    if (ctx->est_scratch) cudaFree(ctx->est_scratch);
     if (ctx->h_est) cudaFreeHost(ctx->h_est);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     cudaEventDestroy(ctx->ev_k0);
@@ -1066,32 +1078,32 @@ int estimator_reduce(ising_ctx* ctx, const int64_t* work_int, int n_traj, double
         src = (const long long*)ctx->est_in.ptr;
     }
     const int B = n_jack_bins < n_traj ? n_jack_bins : n_traj;
-    // The grid's scratch (8 KB) and the pinned words its last CTA writes the
-    // estimate to are allocated on the first call and kept, not charged to the
-    // budget (the jobs' memory is what it bounds); without them the one-CTA
-    // kernel runs and its result is copied.
-    if (!ctx->est_scratch) {
-        if (cudaMalloc(&ctx->est_scratch, jz::kEstScratch) != cudaSuccess) {
-            ctx->est_scratch = nullptr;
-            cudaGetLastError();
-        } else if (cudaHostAlloc((void**)&ctx->h_est, 4 * sizeof(double), cudaHostAllocDefault) !=
-                       cudaSuccess ||
-                   cudaMemsetAsync(ctx->est_scratch, 0, jz::kEstScratch, st) != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(ctx->est_scratch);
-            ctx->est_scratch = nullptr;
-        }
+    // The grid's scratch (8 KB, where the budget has room for it) and the pinned
+    // words that its last CTA writes the estimate to are allocated on a context's
+    // first call (105 us at 200 values, later ones 23 us) and kept; without
+    // them the one-CTA kernel runs and its result is copied.
+    if (!ctx->h_est && cudaHostAlloc((void**)&ctx->h_est, kEstBytes, cudaHostAllocDefault) !=
+                           cudaSuccess) {
+        cudaGetLastError();
+        ctx->h_est = nullptr;
     }
+    if (ctx->h_est && ctx->est_out.bytes < kEstGridBytes &&
+        ensure(ctx, ctx->est_out, kEstGridBytes) == ISING_OK &&
+        cudaMemsetAsync(ctx->est_out.ptr, 0, kEstGridBytes, st) != cudaSuccess) {
+        cudaGetLastError();
+        give_back(ctx, ctx->est_out);
+    }
+    if ((rc = ensure(ctx, ctx->est_out, kEstBytes))) return rc;
     const double scale = beta / (double)n_step;
     double h[3];
-    if (ctx->est_scratch) {
+    if (ctx->est_out.bytes >= kEstGridBytes) {
         if ((rc = cuda_err(jz::launch_estimator_grid(src, n_traj, scale, direction, B,
-                                                     ctx->est_scratch, ctx->h_est, st))) ||
+                                                     (char*)ctx->est_out.ptr + 64, ctx->h_est,
+                                                     st))) ||
             (rc = cuda_err(cudaStreamSynchronize(st))))
             return rc;
         std::memcpy(h, ctx->h_est, sizeof h);
     } else {
-        if ((rc = ensure(ctx, ctx->est_out, 4 * sizeof(double)))) return rc;
         if ((rc = cuda_err(jz::launch_estimator(src, n_traj, scale, direction, B,
                                                 (double*)ctx->est_out.ptr, st))) ||
             (rc = cuda_err(cudaMemcpyAsync(h, ctx->est_out.ptr, sizeof h, cudaMemcpyDeviceToHost,

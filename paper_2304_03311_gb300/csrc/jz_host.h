@@ -82,8 +82,10 @@ struct ising_ctx {
     size_t budget = 0;   // 0 = unlimited
     size_t used = 0;
     DevBuf tcut, jobs, work, spins, est_in, est_out;
-    void* est_scratch = nullptr;   // estimator_reduce's partial sums (kEstScratch bytes)
-    double* h_est = nullptr;       // and its result, in pinned memory
+    // est_out: the estimate's words, and where the budget has room the partial sums of
+    // estimator_reduce's grid, given back when it has none left for another buffer;
+    // h_est: the grid's result, in pinned memory
+    double* h_est = nullptr;
     DevBuf lattice;   // HBM lattices of shapes too large for shared memory
     DevBuf therm;     // spins after Swendsen-Wang thermalisation (therm_update = 1)
     std::vector<uint32_t> h_tcut;
