@@ -45,8 +45,9 @@ size_t sw_smem_bytes(const Geom& g);
 // Threads of one Swendsen-Wang CTA (one trajectory) for dimension D.
 int sw_cta_threads(int D);
 // Trajectories one launch of the HBM Swendsen-Wang variant keeps resident on
-// the device at once (its occupancy x SMs): the chunk in which lattices beyond
-// shared memory are thermalised, so that their HBM state stays one wave.
+// the device at once (the CTAs per SM that its registers allow x SMs): the chunk in
+// which lattices beyond shared memory are thermalised, so that their HBM state stays
+// one wave.
 long long sw_hbm_wave(int D);
 // gS: nullptr to keep each trajectory's state in shared memory, else an HBM
 // buffer of n_cta * sw_smem_bytes(g) bytes, one slice per CTA.

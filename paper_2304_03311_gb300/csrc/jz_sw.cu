@@ -543,7 +543,13 @@ using SwFn = void (*)(const SwGeom, const PhiloxKeys, const JobDesc*, int, uint3
 // fit (3 in 3D, 5 in 2D), but in 3D 64 registers without spills when two per SM
 // hold the whole launch anyway (L = 48, L_t = 192, 256 trajectories: 171 ms
 // against 190 ms; 456 trajectories of L = 40, L_t = 80: 68 ms against 49 ms).
+// In 2D the compiler's own 48 registers without spills let five share an SM; asked for
+// five, it takes 48 too, but 1.05 .. 1.08 of the time (L = 192, 760 cluster starts of 20
+// sweeps: 21.3 against 19.7 ms; 28.8 ms before the grouped bond phase).
+//
+// kHbmCtas*: the CTAs per SM that a wave of HBM states counts on (sw_hbm_wave).
 constexpr int kGroupMin = 6;
+constexpr int kHbmCtas2d = 5, kHbmCtas3d = 3;
 static SwFn pick_sw(int D, bool hbm, bool group, long long n_cta)
 {
     if (!hbm && D == 3)
@@ -555,16 +561,17 @@ static SwFn pick_sw(int D, bool hbm, bool group, long long n_cta)
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         n_cta <= 2LL * n_sm)
         return sw_kernel<3, true, true, 2>;
-    return sw_kernel<3, true, true, 3>;
+    return sw_kernel<3, true, true, kHbmCtas3d>;
 }
 
 int sw_cta_threads(int D) { return sw_threads(D); }
 
-// Their register counts (40 and 48) let 3 and 5 CTAs share an SM.  Not asked of
-// the runtime, which would load both kernels when a server starts.
+// What the kernels' registers allow: 40 in 3D, by its launch bounds, 48 in 2D, held by
+// a test of the assembler's report.  Not asked of the runtime, which would load both
+// kernels when a server starts.  With fewer resident a wave would only take longer.
 long long sw_hbm_wave(int D)
 {
-    const int per_sm = D == 3 ? 3 : 5;
+    const int per_sm = D == 3 ? kHbmCtas3d : kHbmCtas2d;
     int dev = 0, n_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
