@@ -1328,6 +1328,13 @@ double team_time(const jz::Geom& g, const jz::LaunchShape& sh)
     return jz::sweep_cost(g, sh.team_threads, &kind) + (sh.warp ? 0.0 : 2 * kBarrier);
 }
 
+// The sweeps of a job that the persistent kernel runs: a cluster start's are launches
+// of their own ahead of it.
+double plan_sweeps(const jz_params& p)
+{
+    return (sw_therm(p) ? 0.0 : (double)p.n_therm) + (double)p.n_step * p.n_sweep;
+}
+
 // A job's layout inside the plan's CTAs of cta threads: the warp teams of
 // shape_for, or one team of the whole CTA when that takes less of the CTA's time
 // per trajectory, or when the warp teams' lattices take more than the CTA's share
@@ -1449,8 +1456,7 @@ int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
                      !(sh.warp && sh.cta_threads > cand) && sm <= jz::kMaxSmemPerCta;
                 smem = std::max(smem, sm);
                 pair = pair && jz::traj_pairs(g, sh.teams, false);
-                const double t =
-                    team_time(g, sh) * ((double)p.n_therm + (double)p.n_step * p.n_sweep);
+                const double t = team_time(g, sh) * plan_sweeps(p);
                 const long long c = (p.n_traj + sh.teams - 1) / sh.teams;
                 items.push_back({t, c});
                 sum += t * c;
@@ -1632,8 +1638,7 @@ int plan_build(ising_ctx* ctx, const jz_params* jobs, int n_jobs, int64_t* const
             therm_bytes += (size_t)p.n_traj * (size_t)(B.g.nrep * p.L_t * B.g.Ly * p.L);
             J.start_in = 1;
         }
-        const double time = team_time(B.g, B.sh) *
-                            ((double)p.n_therm + (double)p.n_step * p.n_sweep);
+        const double time = team_time(B.g, B.sh) * plan_sweeps(p);
         for (int lo = 0; lo < p.n_traj; lo += B.sh.teams)
             items.push_back({time, make_int2(j, lo)});
     }
