@@ -196,6 +196,7 @@ int weak_coupling(const jz_params& p)
 }
 
 bool never_flips(const uint32_t tb[4]) { return tb[0] == 0u; }
+bool never_flips(const jz_params& p) { return threshold(2.0 * p.beta * (double)(2 * p.d)) == 0u; }
 
 void build_tables(const jz_params& p, uint32_t tb[4], std::vector<uint32_t>& tcut, size_t off)
 {
@@ -1455,7 +1456,7 @@ int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
                 ok = shape_fits(g) && sh.team_threads <= cand &&
                      !(sh.warp && sh.cta_threads > cand) && sm <= jz::kMaxSmemPerCta;
                 smem = std::max(smem, sm);
-                pair = pair && jz::traj_pairs(g, sh.teams, false);
+                pair = pair && !never_flips(p) && jz::traj_pairs(g, sh.teams, false);
                 const double t = team_time(g, sh) * plan_sweeps(p);
                 const long long c = (p.n_traj + sh.teams - 1) / sh.teams;
                 items.push_back({t, c});

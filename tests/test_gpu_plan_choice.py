@@ -40,3 +40,13 @@ def _job(i, d, L, L_t, n_traj, n_step, n_therm, therm_update=0, beta=None):
 def test_cluster_starts_weigh_what_the_kernel_runs(a, b):
     few, many = (_info([_job(0, *a, 10, n, 1), _job(1, *b, 200, 200)]) for n in (1, 1000000))
     assert few == many
+
+
+def test_strong_couplings_have_no_table():
+    """2D L = 128, L_t = 892: one 114,176 byte lattice per CTA.  Two such CTAs share an
+    SM's 233,472 bytes, with the acceptance table (2 KB each) they do not; jobs whose
+    couplings the table cannot hold run without it, two CTAs of 256 threads per SM."""
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    job = (2, 128, 892, 4 * n_sm, 100, 100)
+    assert _info([_job(0, *job, beta=4.0)])[:2] == (256, 2 * n_sm)
+    assert _info([_job(0, *job)])[1] == n_sm
