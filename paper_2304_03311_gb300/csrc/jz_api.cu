@@ -1420,14 +1420,39 @@ void plan_release(jz_plan* pl)
     delete pl;
 }
 
-// Chooses a plan's CTA size (*cta = 0: open; 0 again if none can run the jobs) and the threads per SM that its layouts make room for: the
-// shortest schedule, each candidate's items handed out as the kernel does, longest
-// first to the CTA that is free first, in shape_score's units (3 warps per SM
-// sub-partition take 0.78 of the time of 4).  27 jobs, 2D L = 32 .. 128 and 3D L = 8
-// .. 24: 49.8 ms with the 384 threads it takes; 55.4 ms with the 256 that a trial
-// run of a sixteenth of the trajectories chose, which saw neither the waves nor
-// the tail of the full plan.  Its 2D L = 96 jobs alone: 13.6 -> 3.8 ms (one team
-// per CTA).
+// The time that `grid` CTAs take for items (time, how many) handed out as the kernel
+// does, longest first to the CTA that is free first.  Once the CTAs' ends lie within
+// one item's time of each other, a round of equal items moves all of them by that time,
+// so whole rounds are added at once.
+double schedule_span(std::vector<std::pair<double, long long>>& items, long long grid)
+{
+    std::sort(items.rbegin(), items.rend());
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    for (long long i = 0; i < grid; ++i) free_at.push(0.0);
+    double rounds = 0.0, span = 0.0;   // ends are rounds + the queue's; span: the last one
+    for (const auto& it : items)
+        for (long long left = it.second; left > 0;) {
+            if (left >= grid && span - free_at.top() <= it.first) {
+                rounds += (double)(left / grid) * it.first;
+                left %= grid;
+                continue;
+            }
+            const double end = free_at.top() + it.first;
+            free_at.pop();
+            free_at.push(end);
+            span = std::max(span, end);
+            --left;
+        }
+    return rounds + span;
+}
+
+// Chooses a plan's CTA size (*cta = 0: open; 0 again if none can run the jobs) and the
+// threads per SM that its layouts make room for: the shortest schedule, in
+// shape_score's units (3 warps per SM sub-partition take 0.78 of the time of 4).  27
+// jobs, 2D L = 32 .. 128 and 3D L = 8 .. 24: 49.8 ms with the 384 threads it takes;
+// 55.4 ms with the 256 that a trial run of a sixteenth of the trajectories chose, which
+// saw neither the waves nor the tail of the full plan.  Its 2D L = 96 jobs alone: 13.6 ->
+// 3.8 ms (one team per CTA).
 int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
 {
     int dev = 0, n_sm = 0;
@@ -1443,7 +1468,6 @@ int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
             std::vector<std::pair<double, long long>> items;   // time, how many
             size_t smem = 0;
             bool ok = true, pair = true;
-            double sum = 0.0;
             long long n = 0;
             for (int j = 0; j < n_jobs && ok; ++j) {
                 const jz_params& p = jobs[j];
@@ -1460,7 +1484,6 @@ int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
                 const double t = team_time(g, sh) * plan_sweeps(p);
                 const long long c = (p.n_traj + sh.teams - 1) / sh.teams;
                 items.push_back({t, c});
-                sum += t * c;
                 n += c;
             }
             if (!ok) continue;
@@ -1471,20 +1494,7 @@ int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
                 continue;
             }
             const long long grid = std::min((long long)per_sm * n_sm, n);
-            double span = sum / grid;
-            if (n <= 20000) {   // beyond that the tail is short
-                std::sort(items.rbegin(), items.rend());
-                std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
-                for (long long i = 0; i < grid; ++i) free_at.push(0.0);
-                span = 0.0;
-                for (const auto& it : items)
-                    for (long long i = 0; i < it.second; ++i) {
-                        const double end = free_at.top() + it.first;
-                        free_at.pop();
-                        free_at.push(end);
-                        span = std::max(span, end);
-                    }
-            }
+            double span = schedule_span(items, grid);
             const int wc = (cand + 31) / 32;
             span *= ((grid + n_sm - 1) / n_sm * wc + 3) / 4 + 0.5;
             if (span < best) {

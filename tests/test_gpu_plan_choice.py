@@ -50,3 +50,9 @@ def test_strong_couplings_have_no_table():
     job = (2, 128, 892, 4 * n_sm, 100, 100)
     assert _info([_job(0, *job, beta=4.0)])[:2] == (256, 2 * n_sm)
     assert _info([_job(0, *job)])[1] == n_sm
+
+
+def test_one_long_trajectory_among_many_short_ones():
+    """30,000 short items, which one team per CTA makes of 30,000 trajectories, do not
+    hide the long one: its team of 512 threads is done first, whatever the others take."""
+    assert _info([_job(0, 2, 128, 128, 1, 100000, 100), _job(1, 2, 20, 20, 30000, 100, 100)])[0] == 512
