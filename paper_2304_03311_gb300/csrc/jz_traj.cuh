@@ -523,28 +523,17 @@ struct Traj {
             if (ODD) x = xshift(p ^= 1);
         };
         int up = 4 * rowW();
-        if constexpr (CLT > 0 && CTS > 2 && CLT % (2 * CTS) == 0) {
-            // two replicas a whole number of bank rows apart: the second one
-            // runs its bulk rows one step later around, so that the two
-            // fall on different banks
+        if constexpr (CLT > 0 && CTS > 2 && CLT % CTS == 0) {
+            // as many rows for every slot, known at compile time: equal passes of at
+            // most six (15 rows: three of five, 2D L = 64 scan 523 ms; 532 in fours
+            // with a remainder, 529 in sevens)
             constexpr int N = CLT / CTS - 1;
-            static_assert(N % 2 == 1, "");
-            if (r0) {
-                p0 += dp;
-                own += stride;
-                o += stride;
-            }
+            constexpr int PASS = N % 6 == 0 ? 6 : N % 5 == 0 ? 5 : N % 4 == 0 ? 4 : N % 3 == 0 ? 3 : 1;
 #pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
+            for (int h = 0; h < N / PASS; ++h) {
 #pragma unroll
-                for (int k = 0; k < N / 2; ++k) row(up);
+                for (int k = 0; k < PASS; ++k) row(up);
             }
-            if (r0) {
-                p0 -= N * dp;
-                own -= N * stride;
-                o -= N * stride;
-            }
-            row(up);
         } else {
             // n_all rows that every slot has, four per pass and then singly,
             // so that a warp's slots do not diverge; then the last row, which
