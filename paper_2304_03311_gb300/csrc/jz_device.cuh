@@ -134,11 +134,11 @@ __host__ __device__ inline RowKind row_kind(const Geom& g, const LaunchShape& sh
     return k;
 }
 
-// A team with a thread per spin word of its lattice, inside a warp.  Where L = 16 in
-// 2D (kernels of compile-time GW = 1), it runs the one-row path (run_rows).
+// A team with a thread per spin word of its lattice.  Where it is a warp team and L =
+// 16 in 2D (kernels of compile-time GW = 1), it runs the one-row path (run_rows).
 __host__ __device__ inline bool one_row_team(const Geom& g, const LaunchShape& sh)
 {
-    return sh.warp && sh.team_threads == g.NR * g.GW;
+    return sh.team_threads == g.NR * g.GW;
 }
 
 // Per-job (one transformation) parameters, device copy.

@@ -166,7 +166,7 @@ cudaError_t launch_traj(int D, const Geom& g, const PhiloxKeys& K, const JobDesc
     // The one-row path counts thresholds itself, for any couplings, and lives in
     // the instantiation with the table (1000 trajectories of 200 sweeps at beta = 3:
     // 0.15 ms, 0.27 ms by the general counting kernel).
-    const bool rows = D == 2 && g.Lh == 8 && one_row_team(g, sh);
+    const bool rows = D == 2 && g.Lh == 8 && sh.warp && one_row_team(g, sh);
     const bool pair = (!never || rows) && traj_pairs(g, sh.teams, hbm);
     const TrajFn kern = select_traj(D, g, sh, hbm, pair);
     const cudaError_t e = open_smem(kern);
