@@ -427,7 +427,7 @@ int estimator_reduce(ising_ctx* ctx, const int64_t* work_int, int n_traj, double
                      double* delta_S2, double* delta_S2_err);
 
 /* Launch-shape control; the paper has no counterpart.  A time slice holds
- * col = ceil(L/8) * L_y spin words; each thread owns one word column of every
+ * col = ceil(L/16) * L_y spin words; each thread owns one word column of every
  * TS-th slice.  Fixes the CTA size the context uses for lattices of shape
  * (d, L, L_t), at most 512 threads:
  *   col <= 32  a multiple of 32: warp teams of col * TS <= 32 threads, as many
@@ -435,9 +435,9 @@ int estimator_reduce(ising_ctx* ctx, const int64_t* work_int, int n_traj, double
  *              fewer than four warp teams' lattices fit its shared memory)
  *   col > 32   col * TS with 1 <= TS <= L_t: one team per CTA
  * threads = 0 restores the default: the shape, among the warp-team layouts of
- * every CTA size and one team per CTA of every TS, that keeps the most lanes
- * of each SM busy for the launch's trajectory count (CUDA occupancy of the
- * kernel that runs the lattice).  Results do not depend on the shape.
+ * every CTA size and one team per CTA of every TS, whose estimated time for the
+ * launch's trajectory count is the shortest (a half-sweep's rows per thread, the
+ * warps that share an SM, the last wave).  Results do not depend on the shape.
  * Errors: ISING_ERR_ARG. */
 int ising_set_threads(ising_ctx* ctx, int d, int L, int L_t, int threads);
 

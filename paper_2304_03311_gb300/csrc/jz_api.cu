@@ -396,8 +396,8 @@ jz::LaunchShape default_shape(int d, const jz::Geom& g, long long n_traj)
     if (col <= 32)
         for (int t = 32; t <= 512; t *= 2) consider(shape_for(g, t));
     // one team per CTA: for w = 1 .. 16 warps the largest slice step that
-    // fits them, and the even step below it; a CTA team has at least a warp
-    // of threads (its first eight fill the shared threshold table)
+    // fits them, and the step below it; a team of less than a warp is a warp
+    // team's job
     int last = 0;
     for (int w = 1; w <= 16; ++w) {
         const int top = std::min(32 * w / col, g.Lt);
@@ -665,6 +665,8 @@ int run_group(ising_ctx* ctx, const jz_params* jobs, const std::vector<int>& idx
     } else {
         uint32_t* gS = nullptr;
         if (in_hbm) gS = (uint32_t*)ctx->lattice.ptr;
+        // one job that the acceptance table cannot hold sends its launch to the counts
+        // (2D L = 64 9.96 ms instead of 9.37, 3D L = 16 5.85 ms instead of 5.19)
         bool never = false;
         for (int i = 0; i < n_jobs; ++i) never = never || never_flips(ctx->h_jobs[i].tb);
         if ((rc = cuda_err(jz::launch_traj(p0.d, g, K, (const jz::JobDesc*)ctx->jobs.ptr,

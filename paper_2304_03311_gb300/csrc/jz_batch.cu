@@ -95,12 +95,14 @@ persistent_kernel(const BatchJob* __restrict__ jobs, const int2* __restrict__ it
 
 // ---------------------------------------------------------- batched estimator --
 constexpr int kMaxJackBlocksB = 64;
+constexpr int kEstBatchThreads = 256;
+static_assert(kEstBatchThreads >= kEstFinish, "");
 
 // One CTA per job: ln <e^-W> as a max-shifted log-sum-exp per jackknife block,
 // then the full and leave-one-block-out estimates (Appendix A, eq.
 // Jarzynski_theorem).  out[3j + 0] = ln <e^-W>, [3j + 1] = Delta S_2,
 // [3j + 2] = jackknife error of Delta S_2.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kEstBatchThreads)
 estimator_batch_kernel(const EstJob* __restrict__ jobs, double* __restrict__ out)
 {
     __shared__ double s_max[kMaxJackBlocksB], s_sum[kMaxJackBlocksB];
@@ -161,7 +163,7 @@ cudaError_t launch_persistent(const BatchJob* jobs, const int2* items, int n_ite
 
 cudaError_t launch_estimator_batch(const EstJob* jobs, int n_jobs, double* out, cudaStream_t st)
 {
-    estimator_batch_kernel<<<n_jobs, 256, 0, st>>>(jobs, out);
+    estimator_batch_kernel<<<n_jobs, kEstBatchThreads, 0, st>>>(jobs, out);
     return cudaGetLastError();
 }
 

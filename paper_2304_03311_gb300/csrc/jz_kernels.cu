@@ -13,9 +13,10 @@ namespace jz {
 // (Appendix A, eq. Jarzynski_theorem; blocked jackknife).
 // out[0] = ln <e^-W>, out[1] = Delta S_2, out[2] = jackknife error.
 constexpr int kMaxJackBlocks = 64;
-constexpr int kEstThreads = 160;
+constexpr int kEstThreads = 160, kEstOneCta = 1024;
+static_assert(kEstThreads >= kEstFinish && kEstOneCta >= kEstFinish, "");
 
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kEstOneCta)
 estimator_kernel(const long long* __restrict__ w_int, int n, double scale, int direction,
                  int n_blocks, double* __restrict__ out)
 {
@@ -50,9 +51,10 @@ estimator_kernel(const long long* __restrict__ w_int, int n, double scale, int d
 // and forms the estimates.
 //
 // What bounds it: FP64 exponentials, about 20 FP64 operations each, at two FP64
-// lanes per clock and SM: 16384 of them take one SM 85 us and 128 SMs under 1 us.
-// One value per thread where the SMs allow it.  16384 values, B = 32, whole
-// call: 153 us on one CTA -> 26 us on 128 (kernel about 15 us).
+// lanes per clock and SM: 16384 of them take one SM 85 us and 96 SMs 1 us; then the
+// finish on one CTA and the call.  A chunk holds a value per thread and up to as many
+// again (the chunk count rounds down): 16384 values, B = 32, are 96 CTAs of 170 or 171
+// values on 160 threads.  Whole call: 153 us on one CTA -> 25 us (kernel about 15 us).
 __global__ void __launch_bounds__(kEstThreads)
 estimator_grid_kernel(const long long* __restrict__ w_int, int n, double scale, int direction,
                       int B, int C, double2* part, unsigned int* done, double* __restrict__ out)
@@ -189,11 +191,12 @@ cudaError_t traj_occupancy(int D, const Geom& g, const LaunchShape& sh, int* cta
 cudaError_t launch_estimator(const long long* w_int, int n, double scale, int direction,
                              int n_blocks, double* out, cudaStream_t st)
 {
-    estimator_kernel<<<1, 1024, 0, st>>>(w_int, n, scale, direction, n_blocks, out);
+    estimator_kernel<<<1, kEstOneCta, 0, st>>>(w_int, n, scale, direction, n_blocks, out);
     return cudaGetLastError();
 }
 
-// Chunks per jackknife block: one value per thread up to kEstMaxCtas CTAs.
+// Chunks per jackknife block: as many as hold a value per thread, up to kEstMaxCtas
+// CTAs.
 cudaError_t launch_estimator_grid(const long long* w_int, int n, double scale, int direction,
                                   int n_blocks, void* scratch, double* out, cudaStream_t st)
 {

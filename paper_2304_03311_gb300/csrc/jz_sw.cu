@@ -26,11 +26,13 @@
 //      lattices (fewer than kGroupMin chunks per warp) take.
 //   B2 the recorded bonds, queued per warp and taken 32 at a time, merge
 //      clusters by lock-free union (the larger root is hooked under the
-//      smaller one, so the root of a cluster is its smallest site index);
-//   CD every site finds its root (halving the path it walks) and flips iff the
-//      root's flip bit is set: each cluster flips with probability 1/2, independently of
-//      the others and of its bonds (a ballot assembles 32 sites into one spin
-//      word).
+//      smaller one, so the root of a cluster is its smallest site index; an
+//      atomicMin whose displaced label is joined in turn, as in Komura, Comput.
+//      Phys. Commun. 194 (2015) 54, and Playne and Hawick, IEEE TPDS 29 (2018)
+//      1217);
+//   CD every site finds its root and flips iff the root's flip bit is set: each
+//      cluster flips with probability 1/2, independently of the others and of
+//      its bonds (a ballot assembles 32 sites into one spin word).
 // The cluster partition, hence the minimum-index root of every cluster, does
 // not depend on the order of the unions, so the result is the same bit for bit
 // as a sequential union-find over the same bonds.
@@ -41,7 +43,7 @@
 // root walk of the flip phase, unions that go on from the hooked root's old
 // parent instead of walking anew, and the grouped bond phase (156 -> 99
 // instructions per 32 sites and sweep), the 2D L = 64 scan of 31 x 64
-// trajectories takes 46 ms instead of 69 ms, 2D L = 128 23 ms (37), 3D 16^3 20 ms
+// trajectories takes 47 ms instead of 69 ms, 2D L = 128 23 ms (37), 3D 16^3 20 ms
 // (27), 3D 20^3 8.5 ms (13.3).
 //
 // Termination: a label always points to a site with a smaller or equal index
@@ -114,10 +116,10 @@ struct SpinBits {
     __device__ __forceinline__ uint32_t operator[](int w) const { return sp[w]; }
 };
 
-// Root of a with path halving: every visited node is re-pointed to its
-// grandparent.  A plain store is enough: the new parent is an ancestor of the
-// node, and a hook that a concurrent union made on that node is only ever
-// overwritten after the union has moved on to join the node's old tree.
+// Root of a with path halving, of the plain form's flip phase: every visited node
+// is re-pointed to its grandparent.  No union runs beside it, and a plain store is
+// enough: a label only ever moves to an ancestor, so concurrent walkers still reach
+// the root.
 __device__ __forceinline__ int find_root(volatile int* lab, int a, int V)
 {
     for (;;) {
@@ -467,11 +469,11 @@ sw_kernel(const SwGeom g, const PhiloxKeys K, const JobDesc* __restrict__ jobs, 
         }
         __syncthreads();
         // phase CD: every site flips iff its cluster's root drew a set flip
-        // bit.  The walks halve the paths they take (a label only ever moves
-        // to an ancestor, so concurrent walkers still reach the root), which
-        // shortens the walks of later sites through them: on the 2D L = 64
-        // and 3D 16^3 scans this phase then takes about a third less time
-        // than with read-only walks.
+        // bit.  The grouped form takes straight-line steps, walks on without
+        // writing, and leaves the root in its own site's label, which shortens
+        // the walks of later sites through it (2D L = 64 scan 48.8 -> 46.4 ms
+        // against walks without the steps and the store); the plain form halves
+        // the paths it walks.
         for (int base = warp * 32; base < g.V; base += chunk) {
             const int i = base + lane;
             int f = 0;
@@ -539,7 +541,7 @@ using SwFn = void (*)(const SwGeom, const PhiloxKeys, const JobDesc*, int, uint3
 //
 // Registers.  In shared memory the compiler's own choice (no occupancy asked
 // for) was the fastest: 2D L = 64 scan 48.8 ms, against 54.7, 54.2 and 56.3 ms when
-// sized for 4, 5 and 6 CTAs.  States beyond it wait on memory: as many CTAs as
+// sized for 4, 5 and 6 CTAs (before the flip phase's straight-line steps: 46.6 ms now).  States beyond it wait on memory: as many CTAs as
 // fit (3 in 3D, 5 in 2D), but in 3D 64 registers without spills when two per SM
 // hold the whole launch anyway (L = 48, L_t = 192, 256 trajectories: 171 ms
 // against 190 ms; 456 trajectories of L = 40, L_t = 80: 68 ms against 49 ms).

@@ -38,10 +38,11 @@
 // 1.8, every multiply-add 1.4, every shared load about 1.  So the update is
 // written for few instructions of any kind: thresholds looked up for two sites
 // at once, sums instead of XORs, one funnel shift per word, wrap-free bulk rows.
-// 2D L = 64: 134 instructions and 230 cycles per word (158 and 311 with one
-// lookup per site, four copies of the half-sweep whose code overflowed the
-// instruction cache, and a cut pass that recomputed its geometry): a scan of 31 x
-// 1024 trajectories 761 -> 527 ms, 1.02e12 -> 1.48e12 spin updates/s.
+// 2D L = 64: 130 instructions and 206 cycles per word at the 1.975 GHz that the
+// cycle counter shows under this load (158 and 300 with one lookup per site, four
+// copies of the half-sweep whose code overflowed the instruction cache, and a cut pass
+// that recomputed its geometry): a scan of 31 x 1024 trajectories 761 -> 523 ms,
+// 1.02e12 -> 1.49e12 spin updates/s.
 //
 // The work increment is gathered inside the first colour-0 half-sweep of each
 // step: for every (r, y) exactly one of the switched sites (l, y, 0)^r and
@@ -721,7 +722,7 @@ struct Course {
 // Philox blocks and counts their thresholds (neither depends on spins) beside
 // its own update, both colours' own words stay in registers, and everything of
 // rounds 0 to 2 that does not depend on the sweep is computed once.
-template <bool FAST, class Tr, class Bar>
+template <class Tr, class Bar>
 __device__ __forceinline__ int run_rows(const Tr& tr, const Geom& g, const PhiloxKeys& K,
                                         const TeamJob& J, Bar bar)
 {
@@ -845,7 +846,7 @@ __device__ __forceinline__ int run_trajectory(const Geom& g, const PhiloxKeys& K
     }
     bar();
     if constexpr (ROW) {
-        return run_rows<KIND == kWhole>(tr, g, K, J, bar);
+        return run_rows(tr, g, K, J, bar);
     } else {
         int dE = 0;
         Course<D> C(J);
