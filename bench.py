@@ -290,7 +290,7 @@ KERNEL_SOURCES = {
     "traj_kernel": ("jz_traj2d.cu", "jz_traj3d.cu", "jz_traj_kernel.cuh", "jz_traj.cuh",
                     "jz_device.cuh"),
     "persistent_kernel": ("jz_batch.cu", "jz_traj.cuh", "jz_device.cuh"),
-    "sw_kernel": ("jz_sw.cu", "jz_device.cuh"),
+    "sw_kernel": ("jz_sw.cu", "jz_sw_words.cuh", "jz_device.cuh"),
 }
 
 

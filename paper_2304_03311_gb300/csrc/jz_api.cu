@@ -1451,8 +1451,8 @@ double schedule_span(std::vector<std::pair<double, long long>>& items, long long
 // Chooses a plan's CTA size (*cta = 0: open; 0 again if none can run the jobs) and the
 // threads per SM that its layouts make room for: the shortest schedule, in
 // shape_score's units (3 warps per SM sub-partition take 0.78 of the time of 4).  27
-// jobs, 2D L = 32 .. 128 and 3D L = 8 .. 24: 49.8 ms with the 384 threads it takes;
-// 55.4 ms with the 256 that a trial run of a sixteenth of the trajectories chose, which
+// jobs, 2D L = 32 .. 128 and 3D L = 8 .. 24: 49.8 ms with the 384 threads it takes
+// (48.6 ms with the present kernels); 55.4 ms with the 256 that a trial run of a sixteenth of the trajectories chose, which
 // saw neither the waves nor the tail of the full plan.  Its 2D L = 96 jobs alone: 13.6 ->
 // 3.8 ms (one team per CTA).
 int plan_cta(const jz_params* jobs, int n_jobs, int* cta, int* resident)
