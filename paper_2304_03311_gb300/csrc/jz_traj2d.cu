@@ -6,7 +6,8 @@ namespace jz {
 // Shapes with compile-time row geometry: L = 16 and 64 (GW = 1, 4); the L =
 // L_t = 64 warp teams of an even number of replicas also fix L_t and the slice step
 // (four slices by two replicas at a time; 31 x 1024 trajectories 533 ms with eight
-// slices of one, 527 so, 523 with the present passes).  Every other shape runs the generic instantiation.
+// slices of one, 527 so, 523 with the present passes).  Every other shape runs the
+// generic instantiation.
 TrajFn select_traj2d(const Geom& g, const LaunchShape& sh, bool hbm, bool pair)
 {
     const int kind = row_kind(g, sh);
