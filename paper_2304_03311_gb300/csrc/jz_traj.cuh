@@ -38,11 +38,10 @@
 // 1.8, every multiply-add 1.4, every shared load about 1.  So the update is
 // written for few instructions of any kind: thresholds looked up for two sites
 // at once, sums instead of XORs, one funnel shift per word, wrap-free bulk rows.
-// 2D L = 64: 130 instructions and 206 cycles per word at the 1.975 GHz that the
-// cycle counter shows under this load (158 and 300 with one lookup per site, four
-// copies of the half-sweep whose code overflowed the instruction cache, and a cut pass
-// that recomputed its geometry): a scan of 31 x 1024 trajectories 761 -> 523 ms,
-// 1.02e12 -> 1.49e12 spin updates/s.
+// 2D L = 64: 130 instructions and 216 cycles per word (158 and 314 with one lookup per
+// site, four copies of the half-sweep whose code overflowed the instruction cache, and a
+// cut pass that recomputed its geometry): a scan of 31 x 1024 trajectories 761 -> 523 ms,
+// 1.02e12 -> 1.49e12 spin updates/s, at 2.07 GHz.
 //
 // The work increment is gathered inside the first colour-0 half-sweep of each
 // step: for every (r, y) exactly one of the switched sites (l, y, 0)^r and
